@@ -17,84 +17,11 @@
 #include "../../include/vdi.h"
 #include "vdi_api_internal.h"
 #include "vdi_internal.cuh"
+#include "vdi_sample.cuh"
 
 namespace vdi {
 
 constexpr long long kMaxSamples = 1 << 22;  // per ray; the host rejects steps that would need more
-
-struct GenConsts {
-    float E[3], D0[3], Dx[3], Dy[3];  // ray p(t) = E + t (D0 + x Dx + y Dy), t = V_O view depth
-    float t_near, t_far, P22, P23;    // NDC z = P23 / t - P22
-    float bmin[3], bmax[3], ext[3];
-    float step, u, tau, adj_exp;
-    int step_is_u;
-    float kv[16], kc[16][4];
-    int nk;
-    int w, h, ns, nsp;
-    long long nl;
-    int nx, ny, nz, dtype;
-    const void *data;
-    int fmt;
-    int adaptive;  // 1: per-ray gamma by Algorithm 3 (tau unused)
-};
-
-#define ADD __fadd_rn
-#define SUB __fsub_rn
-#define MUL __fmul_rn
-#define DIV __fdiv_rn
-
-__device__ __forceinline__ float lerp_rn(float a, float b, float t) { return ADD(a, MUL(t, SUB(b, a))); }
-
-__device__ __forceinline__ float voxel(const GenConsts &g, int i, int j, int k) {
-    const size_t o = ((size_t)k * g.ny + j) * g.nx + i;
-    if (g.dtype == 0) return DIV((float)__ldg(reinterpret_cast<const uint8_t *>(g.data) + o), 255.f);
-    if (g.dtype == 1) return DIV((float)__ldg(reinterpret_cast<const uint16_t *>(g.data) + o), 65535.f);
-    return __ldg(reinterpret_cast<const float *>(g.data) + o);
-}
-
-__device__ __forceinline__ float trilinear(const GenConsts &g, const float p[3]) {
-    const int n[3] = {g.nx, g.ny, g.nz};
-    int i0[3], i1[3];
-    float fr[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const float q = SUB(MUL(DIV(SUB(p[c], g.bmin[c]), g.ext[c]), (float)n[c]), 0.5f);
-        const float fl = floorf(q);
-        fr[c] = SUB(q, fl);
-        const int i = (int)fl;
-        i0[c] = min(max(i, 0), n[c] - 1);
-        i1[c] = min(max(i + 1, 0), n[c] - 1);
-    }
-    const float c00 = lerp_rn(voxel(g, i0[0], i0[1], i0[2]), voxel(g, i1[0], i0[1], i0[2]), fr[0]);
-    const float c10 = lerp_rn(voxel(g, i0[0], i1[1], i0[2]), voxel(g, i1[0], i1[1], i0[2]), fr[0]);
-    const float c01 = lerp_rn(voxel(g, i0[0], i0[1], i1[2]), voxel(g, i1[0], i0[1], i1[2]), fr[0]);
-    const float c11 = lerp_rn(voxel(g, i0[0], i1[1], i1[2]), voxel(g, i1[0], i1[1], i1[2]), fr[0]);
-    return lerp_rn(lerp_rn(c00, c10, fr[1]), lerp_rn(c01, c11, fr[1]), fr[2]);
-}
-
-__device__ __forceinline__ void classify(const GenConsts &g, float v, float out[4]) {
-    const int last = g.nk - 1;
-    if (v <= g.kv[0]) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) out[c] = g.kc[0][c];
-        return;
-    }
-    if (v >= g.kv[last]) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) out[c] = g.kc[last][c];
-        return;
-    }
-    int i = 0;
-    while (i < last - 1 && !(v < g.kv[i + 1])) ++i;
-    const float s = DIV(SUB(v, g.kv[i]), SUB(g.kv[i + 1], g.kv[i]));
-#pragma unroll
-    for (int c = 0; c < 4; ++c) out[c] = lerp_rn(g.kc[i][c], g.kc[i + 1][c], s);
-}
-
-struct SegWriter {
-    float pf, pb;      // pending even slot (depth)
-    float4 pc;         // pending even slot (colour)
-};
 
 __device__ __forceinline__ unsigned h2bits(float a, float b) {
     __half2 h = __floats2half2_rn(a, b);
@@ -162,104 +89,183 @@ __device__ __forceinline__ GenRay gen_ray(const GenConsts &g, int px, int py) {
     return r;
 }
 
-// One march along the ray with sensitivity tau (Eq. 1).  WRITE: supersegments
-// go to the VDI, the N_S-th never closes, returns how many were written.
-// !WRITE (the counting pass of Algorithm 3): no limit on the number, nothing
-// written, and the count stops at ns + 1 ("more than N_S").
+// Eq. 1 over a ray's samples, in order: the running mean and composite of the
+// open supersegment, and the closed ones.  WRITE: supersegments go to the VDI,
+// the N_S-th never closes.  !WRITE (the counting pass of Algorithm 3): no
+// limit on the number, nothing written, and the count stops at ns + 1 ("more
+// than N_S").  Sample k covers the ray parameters t0 + k dt .. t0 + (k + 1) dt.
 template <bool WRITE>
-__device__ int gen_march(const GenConsts &g, const GenRay &r, float tau, float4 *__restrict__ depth,
-                         void *__restrict__ colour, long long li, float &first_f, float &last_b) {
-    const int limit = WRITE ? g.ns : g.ns + 2;  // supersegment number `limit` never closes
-    int nseg = 0;
-    SegWriter sw;
-    sw.pf = sw.pb = INFINITY;
-    sw.pc = make_float4(0.f, 0.f, 0.f, 0.f);
-    bool open = false;
-    float t_start = 0.f, t_end = 0.f, Tseg = 1.f, Tray = 1.f;
-    float mean[3] = {0.f, 0.f, 0.f}, Cacc[3] = {0.f, 0.f, 0.f};
-    int cnt = 0;
-    const float tau2 = MUL(tau, tau);
-    auto close = [&]() {
+struct Merger {
+    float tau2;
+    int nseg, cnt;
+    bool open;
+    float fcnt, mean[3];
+    float C[3], T, k_start, k_end;   // open supersegment: composite, transmittance, first and end sample
+    float pf, pb;                    // pending even slot
+    float4 pc;
+    float first_f, last_b;
+
+    __device__ __forceinline__ void begin(float tau) {
+        tau2 = MUL(tau, tau);
+        nseg = cnt = 0;
+        open = false;
+        fcnt = 0.f;
+        T = 1.f;
+        k_start = k_end = 0.f;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) mean[c] = C[c] = 0.f;
+        pf = pb = first_f = INFINITY;
+        last_b = -INFINITY;
+        pc = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+
+    __device__ __forceinline__ void close(const GenConsts &g, const GenRay &r, float4 *depth, void *colour,
+                                          long long li) {
         if (WRITE) {
+            const float t_start = ADD(r.t0, MUL(k_start, r.dt)), t_end = ADD(r.t0, MUL(k_end, r.dt));
             const float f = SUB(DIV(g.P23, t_start), g.P22);
             const float b = SUB(DIV(g.P23, t_end), g.P22);
-            const float aacc = 1.f - Tseg;
+            const float aacc = 1.f - T;
             const float Lu = (t_end - t_start) * r.len / g.u;  // world length in length units
             const float ia = aacc > 0.f ? 1.f / aacc : 0.f;
-            const float kappa = (Lu > 0.f) ? -log2f(Tseg) / Lu : 0.f;
-            const float4 col =
-                make_float4(fminf(Cacc[0] * ia, 1.f), fminf(Cacc[1] * ia, 1.f), fminf(Cacc[2] * ia, 1.f), kappa);
+            const float kappa = (Lu > 0.f) ? -log2f(T) / Lu : 0.f;
+            const float4 col = make_float4(fminf(C[0] * ia, 1.f), fminf(C[1] * ia, 1.f), fminf(C[2] * ia, 1.f), kappa);
             if (nseg == 0) first_f = f;
             last_b = b;
             if ((nseg & 1) == 0) {
-                sw.pf = f;
-                sw.pb = b;
-                sw.pc = col;
+                pf = f;
+                pb = b;
+                pc = col;
             } else {
-                write_pair(g, depth, colour, li, nseg >> 1, sw.pf, sw.pb, sw.pc, f, b, col);
+                write_pair(g, depth, colour, li, nseg >> 1, pf, pb, pc, f, b, col);
             }
         }
         ++nseg;
         open = false;
-    };
-    for (long long k = 0; k < r.K; ++k) {
-        const float fk = (float)k;
-        const float ta = ADD(r.t0, MUL(fk, r.dt));
-        const float tm = ADD(r.t0, MUL(ADD(fk, 0.5f), r.dt));
-        const float tb = ADD(r.t0, MUL((float)(k + 1), r.dt));
-        float p[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) p[c] = ADD(g.E[c], MUL(tm, r.dir[c]));
-        float tf[4];
-        classify(g, trilinear(g, p), tf);
-        const float a = g.step_is_u ? tf[3] : 1.f - powf(1.f - tf[3], g.adj_exp);
-        if (!(a > 0.f)) {
-            if (open && nseg < limit - 1) {
-                close();
-                if (!WRITE && nseg > g.ns) return g.ns + 1;
-            }
-            continue;
+    }
+
+    // supersegments that may close: the last one allowed stays open
+    __device__ __forceinline__ bool may_close(const GenConsts &g) const { return open && nseg < (WRITE ? g.ns - 1 : g.ns + 1); }
+
+    // a transparent sample; true: the count is decided
+    __device__ __forceinline__ bool gap(const GenConsts &g, const GenRay &r, float4 *depth, void *colour, long long li) {
+        if (may_close(g)) {
+            close(g, r, depth, colour, li);
+            if (!WRITE && nseg > g.ns) return true;
         }
-        const float xc[3] = {MUL(tf[0], a), MUL(tf[1], a), MUL(tf[2], a)};
-        if (open && nseg < limit - 1) {
-            const float d0 = SUB(mean[0], xc[0]), d1 = SUB(mean[1], xc[1]), d2 = SUB(mean[2], xc[2]);
-            const float dist2 = ADD(ADD(MUL(d0, d0), MUL(d1, d1)), MUL(d2, d2));
+        return false;
+    }
+
+    // sample k with premultiplied colour (x, y, z) and opacity a > 0; true: the count is decided
+    __device__ __forceinline__ bool add(const GenConsts &g, const GenRay &r, float k, float x, float y, float z, float a,
+                                        float4 *depth, void *colour, long long li) {
+        const float xc[3] = {x, y, z};
+        float e[3];  // sample - mean
+#pragma unroll
+        for (int c = 0; c < 3; ++c) e[c] = SUB(xc[c], mean[c]);
+        if (may_close(g)) {
+            const float dist2 = ADD(ADD(MUL(e[0], e[0]), MUL(e[1], e[1])), MUL(e[2], e[2]));
             if (!(tau2 > dist2)) {
-                close();
-                if (!WRITE && nseg > g.ns) return g.ns + 1;
+                close(g, r, depth, colour, li);
+                if (!WRITE && nseg > g.ns) return true;
             }
         }
         if (!open) {
             open = true;
-            t_start = ta;
             cnt = 0;
-            Tseg = 1.f;
+            fcnt = 0.f;
+            k_start = k;
+            T = 1.f;
 #pragma unroll
-            for (int c = 0; c < 3; ++c) mean[c] = Cacc[c] = 0.f;
+            for (int c = 0; c < 3; ++c) {
+                mean[c] = C[c] = 0.f;
+                e[c] = xc[c];
+            }
         }
         ++cnt;
+        fcnt += 1.f;
+        // mean += (sample - mean) / count: a tabulated reciprocal of the count
+        // (div_by: a quotient small enough to lose its residual lies below
+        // 2^-75, where it changes no squared distance)
+        if (cnt < kRcpTable) {
+            const float rc = __ldg(&kRcp.v[cnt]);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            mean[c] = ADD(mean[c], DIV(SUB(xc[c], mean[c]), (float)cnt));
-            Cacc[c] = ADD(Cacc[c], MUL(Tseg, xc[c]));
+            for (int c = 0; c < 3; ++c) mean[c] = ADD(mean[c], div_by(e[c], fcnt, rc));
+        } else {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) mean[c] = ADD(mean[c], DIV(e[c], fcnt));
         }
-        Tseg = MUL(Tseg, SUB(1.f, a));
-        t_end = tb;
-        Tray = MUL(Tray, SUB(1.f, a));
-        if (Tray <= kErtT) break;
+        if (WRITE) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) C[c] = ADD(C[c], MUL(T, xc[c]));
+            T = MUL(T, SUB(1.f, a));
+            k_end = ADD(k, 1.f);
+        }
+        return false;
     }
-    if (open) close();
-    if (!WRITE) return nseg > g.ns ? g.ns + 1 : nseg;
-    // pad the remaining slots
-    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    int j = nseg;
-    if (j & 1) {
-        write_pair(g, depth, colour, li, j >> 1, sw.pf, sw.pb, sw.pc, INFINITY, INFINITY, zero);
-        ++j;
+
+    // the end of the ray; WRITE: pads the remaining slots
+    __device__ __forceinline__ int finish(const GenConsts &g, const GenRay &r, float4 *depth, void *colour, long long li) {
+        if (open) close(g, r, depth, colour, li);
+        if (!WRITE) return nseg > g.ns ? g.ns + 1 : nseg;
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        int j = nseg;
+        if (j & 1) {
+            write_pair(g, depth, colour, li, j >> 1, pf, pb, pc, INFINITY, INFINITY, zero);
+            ++j;
+        }
+        for (; j < g.nsp; j += 2)
+            write_pair(g, depth, colour, li, j >> 1, INFINITY, INFINITY, zero, INFINITY, INFINITY, zero);
+        return nseg;
     }
-    for (; j < g.nsp; j += 2)
-        write_pair(g, depth, colour, li, j >> 1, INFINITY, INFINITY, zero, INFINITY, INFINITY, zero);
-    return nseg;
+};
+
+// The volume's samples along a ray, in order, until `use(k, tf, a)` returns
+// true or the ray is opaque (transmittance 2^-12).  Two samples' voxels are
+// requested together: they do not depend on what becomes of the first.
+template <int DT, class F>
+__device__ __forceinline__ void sample_ray(const GenConsts &g, const TfTable &tft, const GenRay &r, F use) {
+    constexpr int U = 2;
+    float fk = 0.f, Tray = 1.f;
+    const int K = (int)r.K;
+    for (int k0 = 0; k0 < K; k0 += U) {
+        Voxels<DT> vx[U];
+#pragma unroll
+        for (int i = 0; i < U; ++i) {  // past the ray's last sample: clamped addresses, not used
+            const float tm = ADD(r.t0, MUL(ADD(fk + (float)i, 0.5f), r.dt));
+            float p[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) p[c] = ADD(g.E[c], MUL(tm, r.dir[c]));
+            load_voxels<DT>(g, p, vx[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            if (k0 + i >= K) return;
+            const float v = interpolate<DT>(g, vx[i]);
+            const float4 tf = classify<DT>(g, tft, v);
+            const float a = step_opacity(g, tf.w);
+            if (use(fk + (float)i, v, tf, a)) return;
+            if (a > 0.f) {
+                Tray = MUL(Tray, SUB(1.f, a));
+                if (Tray <= kErtT) return;
+            }
+        }
+        fk += (float)U;
+    }
+}
+
+// One march along the ray with sensitivity tau (Eq. 1); the number of supersegments
+template <int DT, bool WRITE>
+__device__ __forceinline__ int gen_march(const GenConsts &g, const TfTable &tft, const GenRay &r, float tau, Merger<WRITE> &m,
+                                         float4 *depth, void *colour, long long li) {
+    m.begin(tau);
+    bool over = false;
+    sample_ray<DT>(g, tft, r, [&](float k, float, const float4 &tf, float a) {
+        over = a > 0.f ? m.add(g, r, k, MUL(tf.x, a), MUL(tf.y, a), MUL(tf.z, a), a, depth, colour, li)
+                       : m.gap(g, r, depth, colour, li);
+        return over;
+    });
+    return over ? g.ns + 1 : m.finish(g, r, depth, colour, li);
 }
 
 // Ray-adaptive sensitivity (Section 3, Algorithm 3 of the supplement): a
@@ -272,15 +278,16 @@ __device__ int gen_march(const GenConsts &g, const GenRay &r, float tau, float4 
 // that does not exceed N_S).  In [0, sqrt(3)] an FP32 ulp is at most 1.2e-7,
 // so every interval still to be halved holds more than eight ulps and its
 // midpoint lies strictly inside it.  FP32 with explicit rounding, like the
-// march, so every ray's gamma is reproducible.
-__device__ float adaptive_tau(const GenConsts &g, const GenRay &r) {
+// march, so every ray's gamma is reproducible.  count(gamma): the ray's
+// supersegments at gamma, ns + 1 for "more than N_S".
+template <class F>
+__device__ __forceinline__ float adaptive_tau(const GenConsts &g, F count) {
     const int delta = (15 * g.ns) / 100;
     float low = 0.f, high = (float)1.7320508075688772, gamma = (float)1e-5;
     const float eps = (float)1e-6;
     bool first = true, found = false;
-    float ff = 0.f, lb = 0.f;
     while (!found) {
-        const int n = gen_march<false>(g, r, gamma, nullptr, nullptr, 0, ff, lb);
+        const int n = count(gamma);
         if (SUB(high, low) < eps) {
             found = true;
             gamma = high;
@@ -300,18 +307,27 @@ __device__ float adaptive_tau(const GenConsts &g, const GenRay &r) {
     return gamma;
 }
 
+// One ray per thread.
+template <int DT, bool ADAPTIVE>
 __global__ void __launch_bounds__(256) generate_kernel(const GenConsts g, float4 *__restrict__ depth,
                                                        void *__restrict__ colour, float2 *__restrict__ range,
                                                        float *__restrict__ tau_out) {
+    __shared__ TfTable tft;
+    load_tf(g, tft);
     const int px = blockIdx.x * 32 + (threadIdx.x & 31);
     const int py = blockIdx.y * 8 + (threadIdx.x >> 5);
     if (px >= g.w || py >= g.h) return;
     const long long li = (long long)py * g.w + px;
     const GenRay r = gen_ray(g, px, py);
-    const float tau = g.adaptive ? adaptive_tau(g, r) : g.tau;
-    float first_f = INFINITY, last_b = -INFINITY;
-    gen_march<true>(g, r, tau, depth, colour, li, first_f, last_b);
-    range[li] = make_float2(first_f, last_b);
+    float tau = g.tau;
+    if (ADAPTIVE)
+        tau = adaptive_tau(g, [&](float gamma) {
+            Merger<false> m;
+            return gen_march<DT, false>(g, tft, r, gamma, m, nullptr, nullptr, 0);
+        });
+    Merger<true> m;
+    gen_march<DT, true>(g, tft, r, tau, m, depth, colour, li);
+    range[li] = make_float2(m.first_f, m.last_b);
     if (tau_out) tau_out[li] = tau;
 }
 
@@ -321,27 +337,25 @@ __global__ void __launch_bounds__(256) generate_kernel(const GenConsts g, float4
 // the transfer function, a' = 1 - (1 - alpha)^(step / u), early termination
 // at transmittance 2^-12.  It is the ground truth the VDI renders are compared
 // with (Section 6).  One thread per pixel; output premultiplied RGBA.
+template <int DT>
 __global__ void __launch_bounds__(256) dvr_kernel(const GenConsts g, void *__restrict__ out, int out_fmt) {
+    __shared__ TfTable tft;
+    load_tf(g, tft);
     const int px = blockIdx.x * 32 + (threadIdx.x & 31);
     const int py = blockIdx.y * 8 + (threadIdx.x >> 5);
     if (px >= g.w || py >= g.h) return;
     const GenRay r = gen_ray(g, px, py);
     float C[3] = {0.f, 0.f, 0.f}, T = 1.f;
-    for (long long k = 0; k < r.K; ++k) {
-        const float tm = ADD(r.t0, MUL(ADD((float)k, 0.5f), r.dt));
-        float p[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) p[c] = ADD(g.E[c], MUL(tm, r.dir[c]));
-        float tf[4];
-        classify(g, trilinear(g, p), tf);
-        const float a = g.step_is_u ? tf[3] : 1.f - powf(1.f - tf[3], g.adj_exp);
-        if (!(a > 0.f)) continue;
-        const float wgt = MUL(T, a);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) C[c] = ADD(C[c], MUL(wgt, tf[c]));
-        T = MUL(T, SUB(1.f, a));
-        if (T <= kErtT) break;
-    }
+    sample_ray<DT>(g, tft, r, [&](float, float, const float4 &tf, float a) {
+        if (a > 0.f) {
+            const float wgt = MUL(T, a);
+            C[0] = ADD(C[0], MUL(wgt, tf.x));
+            C[1] = ADD(C[1], MUL(wgt, tf.y));
+            C[2] = ADD(C[2], MUL(wgt, tf.z));
+            T = MUL(T, SUB(1.f, a));
+        }
+        return false;
+    });
     const size_t idx = (size_t)py * g.w + px;
     if (out_fmt == 0) {
         reinterpret_cast<float4 *>(out)[idx] = make_float4(C[0], C[1], C[2], 1.f - T);
@@ -354,8 +368,34 @@ __global__ void __launch_bounds__(256) dvr_kernel(const GenConsts g, void *__res
 }
 
 cudaError_t launch_dvr(const GenConsts &g, void *out, int out_fmt, cudaStream_t st) {
-    dim3 grid(div_up(g.w, 32), div_up(g.h, 8));
-    dvr_kernel<<<grid, 256, 0, st>>>(g, out, out_fmt);
+    const dim3 grid(div_up(g.w, 32), div_up(g.h, 8));
+    switch (g.fast ? g.dtype : kGeneral) {
+        case 0: dvr_kernel<0><<<grid, 256, 0, st>>>(g, out, out_fmt); break;
+        case 1: dvr_kernel<1><<<grid, 256, 0, st>>>(g, out, out_fmt); break;
+        case 2: dvr_kernel<2><<<grid, 256, 0, st>>>(g, out, out_fmt); break;
+        default: dvr_kernel<kGeneral><<<grid, 256, 0, st>>>(g, out, out_fmt);
+    }
+    return cudaGetLastError();
+}
+
+template <int DT>
+static void launch_generate_t(const GenConsts &g, bool adaptive, float4 *depth, void *colour, float2 *range, float *tau_out,
+                              cudaStream_t st) {
+    const dim3 grid(div_up(g.w, 32), div_up(g.h, 8));
+    if (adaptive)
+        generate_kernel<DT, true><<<grid, 256, 0, st>>>(g, depth, colour, range, tau_out);
+    else
+        generate_kernel<DT, false><<<grid, 256, 0, st>>>(g, depth, colour, range, tau_out);
+}
+
+static cudaError_t launch_generate(const GenConsts &g, bool adaptive, float4 *depth, void *colour, float2 *range,
+                                   float *tau_out, cudaStream_t st) {
+    switch (g.fast ? g.dtype : kGeneral) {
+        case 0: launch_generate_t<0>(g, adaptive, depth, colour, range, tau_out, st); break;
+        case 1: launch_generate_t<1>(g, adaptive, depth, colour, range, tau_out, st); break;
+        case 2: launch_generate_t<2>(g, adaptive, depth, colour, range, tau_out, st); break;
+        default: launch_generate_t<kGeneral>(g, adaptive, depth, colour, range, tau_out, st);
+    }
     return cudaGetLastError();
 }
 
@@ -430,6 +470,7 @@ static vdi_status make_gen_consts(const vdi_volume *vol, const vdi_tf *tf, const
     g->step_is_u = g->step == g->u;
     g->adj_exp = g->step / g->u;
     g->nk = tf->n_knots;
+    for (int k = 0; k < kMaxKnots; ++k) g->kv[k] = INFINITY;
     for (int k = 0; k < g->nk; ++k) {
         g->kv[k] = tf->knots[5 * k];
         for (int c = 0; c < 4; ++c) g->kc[k][c] = tf->knots[5 * k + 1 + c];
@@ -441,6 +482,26 @@ static vdi_status make_gen_consts(const vdi_volume *vol, const vdi_tf *tf, const
     g->nz = vol->nz;
     g->dtype = vol->dtype;
     g->data = vol->data;
+    // The fast sampling forms (vdi_sample.cuh) need voxel indices below 2^21
+    // per axis and 2^31 in all, extents and segment widths whose reciprocals
+    // and residuals stay clear of under- and overflow, and knots that are 0 or
+    // no smaller than 2^-60 (then v - knot is 0 or above 2^-91 for integer
+    // voxels).  Anything else samples by plain divisions.
+    g->fast = vol->nx < (1 << 21) && vol->ny < (1 << 21) && vol->nz < (1 << 21) &&
+              (double)vol->nx * vol->ny * vol->nz < 2147483648.0;
+    g->unit_ext = 1;
+    for (int k = 0; k < 3; ++k) {
+        if (!(g->ext[k] >= 0x1p-30f && g->ext[k] <= 0x1p60f)) g->fast = 0;
+        if (g->ext[k] != 1.f) g->unit_ext = 0;
+        g->iext[k] = 1.f / g->ext[k];
+    }
+    for (int k = 0; k < g->nk; ++k) {
+        if (g->kv[k] != 0.f && !(fabsf(g->kv[k]) >= 0x1p-60f)) g->fast = 0;
+        if (k > 0) {
+            const float width = g->kv[k] - g->kv[k - 1];
+            if (!(width >= 0x1p-60f && width <= 0x1p60f)) g->fast = 0;
+        }
+    }
     return VDI_OK;
 }
 
@@ -476,12 +537,9 @@ VDI_API vdi_status vdi_generate(vdi_ctx *ctx, const vdi_volume *vol, const vdi_t
     g.nsp = v->dv.nsp;
     g.nl = v->dv.nl;
     g.fmt = d.colour_fmt;
-    g.adaptive = prm->adaptive ? 1 : 0;
     cudaStream_t st = (cudaStream_t)stream;
-    dim3 grid(div_up(d.w, 32), div_up(d.h, 8));
-    generate_kernel<<<grid, 256, 0, st>>>(g, reinterpret_cast<float4 *>(v->depth_mem), v->colour_mem, v->range_mem,
-                                          prm->tau_out);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_generate(g, prm->adaptive != 0, reinterpret_cast<float4 *>(v->depth_mem), v->colour_mem,
+                                    v->range_mem, prm->tau_out, st);
     if (e == cudaSuccess) e = launch_grid(v->dv, v->grid_mem, st);
     if (e == cudaSuccess) e = launch_block_range(v->dv, v->brange_mem, st);
     if (e != cudaSuccess) {
