@@ -53,6 +53,7 @@ struct GenConsts {
     int w, h, ns, nsp;
     long long nl;
     int nx, ny, nz, dtype;
+    uint32_t sz;  // nx ny (fast forms)
     const void *data;
     int fmt;
     int fast;      // 1: extents, volume size and knots inside the fast forms' range
@@ -63,8 +64,6 @@ struct GenConsts {
 #define SUB __fsub_rn
 #define MUL __fmul_rn
 #define DIV __fdiv_rn
-
-__device__ __forceinline__ float lerp_rn(float a, float b, float t) { return ADD(a, MUL(t, SUB(b, a))); }
 
 // RN(x / y) for z = RN(1 / y), nothing under- or overflowing (Markstein)
 __device__ __forceinline__ float div_by(float x, float y, float z) {
@@ -104,6 +103,18 @@ __device__ __forceinline__ void load_tf(const GenConsts &g, TfTable &t) {
     __syncthreads();
 }
 
+// Two samples travel together, one in each half of a float2, so that their
+// loads are in flight together.
+__device__ __forceinline__ float2 both(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return make_float2(ADD(a.x, b.x), ADD(a.y, b.y)); }
+__device__ __forceinline__ float2 addrd2(float2 a, float2 b) { return make_float2(__fadd_rd(a.x, b.x), __fadd_rd(a.y, b.y)); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return make_float2(MUL(a.x, b.x), MUL(a.y, b.y)); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return make_float2(SUB(a.x, b.x), SUB(a.y, b.y)); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    return make_float2(__fmaf_rn(a.x, b.x, c.x), __fmaf_rn(a.y, b.y, c.y));
+}
+__device__ __forceinline__ float2 lerp2(float2 a, float2 b, float2 t) { return add2(a, mul2(t, sub2(b, a))); }
+
 // (r, g, b, alpha per length unit) of scalar v
 template <int DT>
 __device__ __forceinline__ float4 classify(const GenConsts &g, const TfTable &t, float v) {
@@ -124,83 +135,124 @@ __device__ __forceinline__ float4 classify(const GenConsts &g, const TfTable &t,
     else
         s = div_by(x, seg.y, seg.z);
     if (DT >= 2 && (j == 0 || j == g.nk)) s = 0.f;  // v may be infinite there
-    return make_float4(ADD(c.x, MUL(s, d.x)), ADD(c.y, MUL(s, d.y)), ADD(c.z, MUL(s, d.z)), ADD(c.w, MUL(s, d.w)));
+    const float2 lo = add2(make_float2(c.x, c.y), mul2(both(s), make_float2(d.x, d.y)));
+    const float2 hi = add2(make_float2(c.z, c.w), mul2(both(s), make_float2(d.z, d.w)));
+    return make_float4(lo.x, lo.y, hi.x, hi.y);
 }
 
-// One sample's eight voxels as loaded, and the interpolation weights
+// The eight voxels of two samples as loaded (an integer, or a float's bits),
+// and their interpolation weights
 template <int DT>
 struct Voxels {
-    uint32_t raw[8];  // the voxel's integer, or the float's bits
-    float fr[3];
+    uint32_t raw[8][2];
+    float2 fr[3];
 };
 
 template <int DT>
-__device__ __forceinline__ void load_voxels(const GenConsts &g, const float p[3], Voxels<DT> &s) {
+__device__ __forceinline__ uint32_t load_raw(const GenConsts &g, size_t o) {
+    const int dt = DT == kGeneral ? g.dtype : DT;
+    return dt == 0   ? __ldg(reinterpret_cast<const uint8_t *>(g.data) + o)
+           : dt == 1 ? __ldg(reinterpret_cast<const uint16_t *>(g.data) + o)
+                     : __ldg(reinterpret_cast<const uint32_t *>(g.data) + o);
+}
+
+// p[c]: coordinate c of the two samples
+template <int DT>
+__device__ __forceinline__ void load_voxels(const GenConsts &g, const float2 p[3], Voxels<DT> &s) {
     const int n[3] = {g.nx, g.ny, g.nz};
-    int i0[3], i1[3];
+    int i0[3][2], i1[3][2];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        float e = SUB(p[c], g.bmin[c]);
+        float2 e = add2(p[c], both(-g.bmin[c]));
         if (DT == kGeneral) {
-            const float q = SUB(MUL(DIV(e, g.ext[c]), (float)n[c]), 0.5f);
-            const float fl = floorf(q);
-            s.fr[c] = SUB(q, fl);
-            const int i = (int)fl;
-            i0[c] = min(max(i, 0), n[c] - 1);
-            i1[c] = min(max(i + 1, 0), n[c] - 1);
-        } else {
-            if (!g.unit_ext) e = div_by(e, g.ext[c], g.iext[c]);
-            const float q = SUB(MUL(e, (float)n[c]), 0.5f);
-            const float t = __fadd_rd(q, 12582912.f);  // 1.5 2^23 + floor(q), |q| < 2^22
-            s.fr[c] = SUB(q, SUB(t, 12582912.f));
-            const int i = __float_as_int(t) - 0x4B400000;
-            i0[c] = min(max(i, 0), n[c] - 1);
-            i1[c] = min(max(i + 1, 0), n[c] - 1);
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {  // the four voxel rows (y, z)
-        const int jy = (k & 1) ? i1[1] : i0[1], kz = (k & 2) ? i1[2] : i0[2];
-        if (DT == kGeneral) {
-            const size_t row = ((size_t)kz * g.ny + jy) * g.nx;
+            float *fr = &s.fr[c].x;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const size_t o = row + (h ? i1[0] : i0[0]);
-                s.raw[2 * k + h] = g.dtype == 0   ? __ldg(reinterpret_cast<const uint8_t *>(g.data) + o)
-                                   : g.dtype == 1 ? __ldg(reinterpret_cast<const uint16_t *>(g.data) + o)
-                                                  : __ldg(reinterpret_cast<const uint32_t *>(g.data) + o);
+                const float q = SUB(MUL(DIV(h ? e.y : e.x, g.ext[c]), (float)n[c]), 0.5f);
+                const float fl = floorf(q);
+                fr[h] = SUB(q, fl);
+                const int i = (int)fl;
+                i0[c][h] = min(max(i, 0), n[c] - 1);
+                i1[c][h] = min(max(i + 1, 0), n[c] - 1);
             }
         } else {
-            const uint32_t row = ((uint32_t)kz * (uint32_t)g.ny + (uint32_t)jy) * (uint32_t)g.nx;
+            if (!g.unit_ext) {
+                const float2 q = mul2(e, both(g.iext[c]));
+                e = fma2(fma2(q, both(-g.ext[c]), e), both(g.iext[c]), q);  // div_by
+            }
+            const float2 q = add2(mul2(e, both((float)n[c])), both(-0.5f));
+            const float2 t = addrd2(q, both(12582912.f));  // 1.5 2^23 + floor(q), |q| < 2^22
+            s.fr[c] = sub2(q, add2(t, both(-12582912.f)));
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const uint32_t o = row + (uint32_t)(h ? i1[0] : i0[0]);
-                s.raw[2 * k + h] = DT == 0   ? __ldg(reinterpret_cast<const uint8_t *>(g.data) + o)
-                                   : DT == 1 ? __ldg(reinterpret_cast<const uint16_t *>(g.data) + o)
-                                             : __ldg(reinterpret_cast<const uint32_t *>(g.data) + o);
+                const int i = __float_as_int(h ? t.y : t.x) - 0x4B400000;
+                i0[c][h] = __vimin_s32_relu(i, n[c] - 1);  // clamped to 0 .. n - 1 in one instruction
+                i1[c][h] = __viaddmin_s32_relu(i, 1, n[c] - 1);
             }
         }
     }
-}
-
-// the scalar a stored voxel stands for
-template <int DT>
-__device__ __forceinline__ float voxel_value(const GenConsts &g, uint32_t raw) {
-    if (DT == 2) return __uint_as_float(raw);
-    if (DT == kGeneral)
-        return g.dtype == 0 ? DIV((float)raw, 255.f) : g.dtype == 1 ? DIV((float)raw, 65535.f) : __uint_as_float(raw);
-    const float b = SUB(__uint_as_float(0x4B000000u | raw), 8388608.f);
-    return DT == 0 ? __fmaf_rn(b, 0x1.010102p-8f, MUL(b, -0x1.fdfdfep-33f))
-                   : __fmaf_rn(b, 0x1.0001p-16f, MUL(b, 0x1.0001p-48f));
-}
-
-template <int DT>
-__device__ __forceinline__ float interpolate(const GenConsts &g, const Voxels<DT> &s) {
-    float c[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-        c[k] = lerp_rn(voxel_value<DT>(g, s.raw[2 * k]), voxel_value<DT>(g, s.raw[2 * k + 1]), s.fr[0]);
-    return lerp_rn(lerp_rn(c[0], c[1], s.fr[1]), lerp_rn(c[2], c[3], s.fr[1]), s.fr[2]);
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {  // the four voxel rows (y, z)
+            const int jy = (k & 1) ? i1[1][h] : i0[1][h], kz = (k & 2) ? i1[2][h] : i0[2][h];
+            if (DT == kGeneral) {
+                const size_t row = ((size_t)kz * g.ny + jy) * g.nx;
+                s.raw[2 * k][h] = load_raw<DT>(g, row + i0[0][h]);
+                s.raw[2 * k + 1][h] = load_raw<DT>(g, row + i1[0][h]);
+            } else {
+                const uint32_t row = (uint32_t)kz * g.sz + (uint32_t)jy * (uint32_t)g.nx;
+                s.raw[2 * k][h] = load_raw<DT>(g, row + (uint32_t)i0[0][h]);
+                s.raw[2 * k + 1][h] = load_raw<DT>(g, row + (uint32_t)i1[0][h]);
+            }
+        }
+}
+
+// the scalars two stored voxels stand for
+template <int DT>
+__device__ __forceinline__ float2 voxel_value(const GenConsts &g, const uint32_t (&raw)[2]) {
+    if (DT == 2 || (DT == kGeneral && g.dtype == 2)) return make_float2(__uint_as_float(raw[0]), __uint_as_float(raw[1]));
+    if (DT == kGeneral) {
+        const float top = g.dtype == 0 ? 255.f : 65535.f;
+        return make_float2(DIV((float)raw[0], top), DIV((float)raw[1], top));
+    }
+    const float2 b = add2(make_float2(__uint_as_float(0x4B000000u | raw[0]), __uint_as_float(0x4B000000u | raw[1])),
+                                both(-8388608.f));
+    return DT == 0 ? fma2(b, both(0x1.010102p-8f), mul2(b, both(-0x1.fdfdfep-33f)))
+                   : fma2(b, both(0x1.0001p-16f), mul2(b, both(0x1.0001p-48f)));
+}
+
+// Whether both samples' eight voxels are equal (and finite): interpolating them
+// gives that voxel exactly, a + t (a - a) = a.  Two opposite corners are
+// compared first, which settles nearly every cell that varies.
+template <int DT>
+__device__ __forceinline__ bool uniform_cells(const Voxels<DT> &s) {
+    if (((s.raw[0][0] ^ s.raw[7][0]) | (s.raw[0][1] ^ s.raw[7][1])) != 0u) return false;
+    uint32_t x = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+        for (int k = 1; k < 7; ++k) x |= s.raw[0][h] ^ s.raw[k][h];
+        if (DT == 2) x |= (s.raw[0][h] & 0x7f800000u) == 0x7f800000u;
+    }
+    return x == 0u;
+}
+
+// The two samples' scalars; true when both cells are uniform.  Homogeneous
+// regions (empty space, the inside of a material) are common in real volumes:
+// there the interpolation is skipped, and the caller keeps the classification
+// while the scalar repeats.
+template <int DT>
+__device__ __forceinline__ bool interpolate(const GenConsts &g, const Voxels<DT> &s, float2 &v) {
+    if (DT != kGeneral && uniform_cells<DT>(s)) {
+        v = voxel_value<DT>(g, s.raw[0]);
+        return true;
+    }
+    float2 c[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) c[k] = lerp2(voxel_value<DT>(g, s.raw[2 * k]), voxel_value<DT>(g, s.raw[2 * k + 1]), s.fr[0]);
+    v = lerp2(lerp2(c[0], c[1], s.fr[1]), lerp2(c[2], c[3], s.fr[1]), s.fr[2]);
+    return false;
 }
 
 // opacity of a sample: alpha of one length unit, or of the sampling step

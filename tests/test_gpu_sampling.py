@@ -75,3 +75,36 @@ def test_generation_decisions_match_oracle(V, ctx, orc, dtype, dims, box, knots,
     valid = np.arange(ns)[None, None, :] < counts[:, :, None]
     assert np.array_equal(g_depth[valid].view(np.uint32), depth[valid].view(np.uint32))
     assert np.abs(g_rgba[valid] - rgba[valid]).max() < 2e-5  # as the existing generation tests
+
+
+@pytest.mark.parametrize("dtype", [np.uint8, np.uint16, np.float32])
+@pytest.mark.parametrize("form", ["recorded", "few rays", "empty", "general", "deep"])
+def test_adaptive_forms_match_oracle(V, ctx, orc, dtype, form):
+    """Algorithm 3 from recorded samples (whole and ragged tiles, rays without a
+    sample), and its two other routes: general sampling, and rays of so many
+    samples (14,000) that they are not recorded.  Gamma, counts and depths are
+    the oracle's."""
+    w, h = {"few rays": (3, 2), "deep": (16, 9)}.get(form, (45, 27))
+    ns, steps = 7, 8200 if form == "deep" else 40
+    bmin, bmax = np.zeros(3), np.ones(3)
+    vol, kn = make_volume(dtype, (24, 20, 28), 5), make_knots(4, 1e-30 if form == "general" else 0.2)
+    if form == "empty":
+        vol[:] = 0
+    if form == "deep":
+        kn[:, 4] *= 0.01
+    u = 1.0 / steps
+    cam = S.orbit_camera(bmin, bmax, w / h, az_deg=30, el_deg=20)
+    args = (kn, cam.view, cam.proj, w, h, ns, 0.0, u, u)
+    rgba, depth, counts, tau = orc.generate(orc.Volume(vol, bmin, bmax), *args, fp32=True, adaptive=True, with_tau=True)
+    t = torch.zeros((h, w), dtype=torch.float32, device="cuda")
+    g = V.vdi_generate(ctx, torch.from_numpy(vol).cuda(), bmin, bmax, kn, V.camera(cam.view, cam.proj), w, h, ns, 0.0, u, u,
+                       V.VDI_F32, adaptive=True, tau_out=t)
+    try:
+        g_rgba, g_depth, g_counts, _ = V.vdi_download(g, w, h, ns)
+    finally:
+        V.vdi_destroy(g)
+    assert (counts.sum() == 0) == (form == "empty")
+    assert np.array_equal(t.cpu().numpy(), tau.reshape(h, w))
+    assert np.array_equal(g_counts, counts)
+    valid = np.arange(ns)[None, None, :] < counts[:, :, None]
+    assert np.array_equal(g_depth[valid].view(np.uint32), depth[valid].view(np.uint32))
