@@ -29,10 +29,9 @@ cudaError_t launch_search(const DevVdi &v, int li, int search, const float *de, 
                           const int32_t *seed, const int32_t *inc, int32_t *res, int n, cudaStream_t st);
 cudaError_t launch_count_leading(const float *depth, int ns, long long nl, int32_t *counts, cudaStream_t st);
 cudaError_t launch_convert(int fmt, const float *rgba, const float *depth, const int32_t *counts, int ns,
-                           int nsp, long long nl, float4 *dpair, void *colour, unsigned *err, cudaStream_t st);
-cudaError_t launch_grid(const DevVdi &v, uint32_t *grid, cudaStream_t st);
-cudaError_t launch_range(const float *depth, const int32_t *counts, int ns, long long nl, float2 *range,
-                         cudaStream_t st);
+                           int nsp, long long nl, float4 *dpair, void *colour, float2 *range, unsigned *err,
+                           cudaStream_t st);
+cudaError_t launch_grid(const DevVdi &v, uint32_t *grid, float2 *brange, cudaStream_t st);
 cudaError_t launch_download(const DevVdi &v, int ns, float *rgba, float *depth, int32_t *counts,
                             cudaStream_t st);
 cudaError_t launch_count_totals(const uint32_t *lists, const uint32_t *segs, long long n, unsigned long long *totals,
@@ -603,6 +602,7 @@ VDI_API vdi_status vdi_create(vdi_ctx *ctx, const vdi_desc *desc, const float *r
     const size_t nl = (size_t)desc->w * desc->h, nslot = nl * desc->n_s;
     float *d_rgba = nullptr, *d_depth = nullptr;
     int32_t *d_counts = nullptr;
+    const int32_t *use_counts = counts;  // device counts are read where they are
     unsigned *d_err = nullptr;
     unsigned h_err = 0;
     if (mem_kind == VDI_MEM_HOST) {
@@ -614,19 +614,19 @@ VDI_API vdi_status vdi_create(vdi_ctx *ctx, const vdi_desc *desc, const float *r
         d_rgba = const_cast<float *>(rgba);
         d_depth = const_cast<float *>(depth);
     }
-    CK(cudaMallocAsync((void **)&d_counts, nl * sizeof(int32_t), st));
     CK(cudaMallocAsync((void **)&d_err, sizeof(unsigned), st));
     CK(cudaMemsetAsync(d_err, 0, sizeof(unsigned), st));
-    if (counts)
-        CK(cudaMemcpyAsync(d_counts, counts, nl * sizeof(int32_t),
-                           mem_kind == VDI_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, st));
-    else
-        CK(launch_count_leading(d_depth, desc->n_s, (long long)nl, d_counts, st));
-    CK(launch_convert(desc->colour_fmt, d_rgba, d_depth, d_counts, desc->n_s, v->dv.nsp, (long long)nl,
-                      reinterpret_cast<float4 *>(v->depth_mem), v->colour_mem, d_err, st));
-    CK(launch_grid(v->dv, v->grid_mem, st));
-    CK(launch_range(d_depth, d_counts, desc->n_s, (long long)nl, v->range_mem, st));
-    CK(launch_block_range(v->dv, v->brange_mem, st));
+    if (!counts || mem_kind == VDI_MEM_HOST) {
+        CK(cudaMallocAsync((void **)&d_counts, nl * sizeof(int32_t), st));
+        use_counts = d_counts;
+        if (counts)
+            CK(cudaMemcpyAsync(d_counts, counts, nl * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+        else
+            CK(launch_count_leading(d_depth, desc->n_s, (long long)nl, d_counts, st));
+    }
+    CK(launch_convert(desc->colour_fmt, d_rgba, d_depth, use_counts, desc->n_s, v->dv.nsp, (long long)nl,
+                      reinterpret_cast<float4 *>(v->depth_mem), v->colour_mem, v->range_mem, d_err, st));
+    CK(launch_grid(v->dv, v->grid_mem, v->brange_mem, st));
     CK(cudaMemcpyAsync(&h_err, d_err, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     if (h_err & 1u)

@@ -56,7 +56,6 @@ cudaError_t launch_render(const ViewConsts &c, const DevVdi &v, void *out, int o
                           cudaStream_t st);
 // the VDI's tensor maps for launch_render, or null when it has none
 inline const TileMaps *tile_maps(const vdi_t *v) { return v->maps_ok ? &v->maps : nullptr; }
-cudaError_t launch_block_range(const DevVdi &v, float2 *brange, cudaStream_t st);
 
 // warp shape used when the caller does not choose one: 4 x 8 pixels per warp
 // (lanes whose rays cross neighbouring lists together), except for exact

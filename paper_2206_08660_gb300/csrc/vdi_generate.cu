@@ -730,7 +730,7 @@ static cudaError_t launch_generate(const GenConsts &g, bool adaptive, double dia
 #undef MUL
 #undef DIV
 
-cudaError_t launch_grid(const DevVdi &v, uint32_t *grid, cudaStream_t st);
+cudaError_t launch_grid(const DevVdi &v, uint32_t *grid, float2 *brange, cudaStream_t st);
 
 }  // namespace vdi
 
@@ -869,8 +869,7 @@ VDI_API vdi_status vdi_generate(vdi_ctx *ctx, const vdi_volume *vol, const vdi_t
     for (int k = 0; k < 3; ++k) diag += (vol->bbox_max[k] - vol->bbox_min[k]) * (vol->bbox_max[k] - vol->bbox_min[k]);
     cudaError_t e = launch_generate(g, prm->adaptive != 0, sqrt(diag), ctx->sm_count, reinterpret_cast<float4 *>(v->depth_mem),
                                     v->colour_mem, v->range_mem, prm->tau_out, st);
-    if (e == cudaSuccess) e = launch_grid(v->dv, v->grid_mem, st);
-    if (e == cudaSuccess) e = launch_block_range(v->dv, v->brange_mem, st);
+    if (e == cudaSuccess) e = launch_grid(v->dv, v->grid_mem, v->brange_mem, st);
     if (e != cudaSuccess) {
         cudaStreamSynchronize(st);
         free_vdi(v);
