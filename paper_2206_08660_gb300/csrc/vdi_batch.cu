@@ -116,13 +116,12 @@ __global__ void __launch_bounds__(256, 4) batch_render_kernel(const BatchParams 
         const int px = tx0 + lx, py = ty0 + ly;
         if (px < q.c.W && py < q.c.H) {
             Accum acc = {0.f, 0.f, 0.f, 1.f};
-            uint32_t nl = 0, nsg = 0;
             Ray ray;
             if (setup_ray(q.c, px, py, v.w, v.h, ray)) {
                 if (v.fmt == 0)
-                    march_exact<0, kSearchAlg2, true>(v, ray, acc, nl, nsg);
+                    march_lists<0>(v, ray, acc);
                 else
-                    march_exact<1, kSearchAlg2, true>(v, ray, acc, nl, nsg);
+                    march_lists<1>(v, ray, acc);
             }
             store_px(q.out, q.out_fmt, (size_t)py * q.c.W + px, acc);
         }

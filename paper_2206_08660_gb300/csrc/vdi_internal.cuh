@@ -124,6 +124,9 @@ struct PairCache {
 __device__ __forceinline__ float4 ld_depth_pair(const DevVdi &v, int k, int li) {
     return __ldg(v.depth + (k * v.nl32 + li));
 }
+__device__ __forceinline__ uint4 ld_colour_pair(const DevVdi &v, int k, int li) {  // FP16 colour
+    return __ldg(reinterpret_cast<const uint4 *>(v.colour) + (k * v.nl32 + li));
+}
 __device__ __forceinline__ float ld_back(const DevVdi &v, int j, int li) {
     const float *p = reinterpret_cast<const float *>(v.depth + ((j >> 1) * v.nl32 + li));
     return __ldg(p + 2 * (j & 1) + 1);

@@ -71,3 +71,42 @@ def test_grid_and_block_ranges(V, ctx, orc, w, h, ns, T, nz, device):
             assert torch.equal(img[0], img[1])
         finally:
             V.vdi_destroy(vdi)
+
+
+@pytest.mark.parametrize("w, h, ns, fmt", [(1, 1, 1, 0), (40, 24, 2, 1), (67, 41, 3, 0), (33, 65, 20, 1), (16, 9, 64, 0)])
+def test_walk_equals_the_searching_walk(V, ctx, w, h, ns, fmt):
+    """The exact frame's walk (seed pair, neighbouring pair, then a search; 16 or
+    32 rays per warp by launch size) against the walk that searches every list
+    from scratch: the same image, bit for bit, for depth rising and falling
+    along the rays, boxes that leave the frustum, and images of one tile, of few
+    and of many."""
+    case = random_case(w, h, ns, seed=w * ns)
+    vdi = V.vdi_create(ctx, case.gpu_desc(V, fmt), case.vdi.rgba, case.vdi.depth, case.vdi.counts)
+    try:
+        for W, H, az, el, zoom in ((1, 1, 20, 0, 1.0), (31, 9, 2, 15, 1.0), (200, 150, 35, -20, 1.0), (640, 400, 100, 30, 1.5),
+                                   (500, 333, 178, 10, 1.0)):
+            cn = S.orbit_camera(case.bmin, case.bmax, W / H, az_deg=az, el_deg=el, zoom=zoom)
+            img = [torch.zeros((H, W, 4), device="cuda") for _ in range(2)]
+            for out, search in zip(img, (V.VDI_SEARCH_ALG2, V.VDI_SEARCH_BINARY)):
+                V.vdi_render_ex(vdi, V.camera(cn.view, cn.proj), W, H, 1, 1, out, search=search)
+            assert torch.equal(img[0], img[1]), (W, H, az)
+    finally:
+        V.vdi_destroy(vdi)
+
+
+@pytest.mark.parametrize("w, h, ns, fmt", [(40, 24, 2, 1), (67, 41, 5, 0), (33, 65, 33, 1)])
+def test_preview_rays_per_warp(V, ctx, w, h, ns, fmt):
+    """Previews at the sizes where the rays per warp change (8, 16, 32 in a launch
+    of its own, 16 in a batch): the same image, bit for bit."""
+    case = random_case(w, h, ns, seed=w)
+    vdi = V.vdi_create(ctx, case.gpu_desc(V, fmt), case.vdi.rgba, case.vdi.depth, case.vdi.counts)
+    try:
+        for W, H in ((5, 3), (40, 30), (800, 600), (1601, 903)):
+            cn = S.orbit_camera(case.bmin, case.bmax, W / H, az_deg=30, el_deg=15)
+            cam = V.camera(cn.view, cn.proj)
+            img = [torch.zeros((H, W, 4), device="cuda") for _ in range(2)]
+            V.vdi_render(vdi, cam, W, H, 1, 2, img[0])
+            V.vdi_render_batch(ctx, [V.request(vdi, cam, W, H, 1, 2, img[1])])
+            assert img[0][..., 3].max() > 0 and torch.equal(img[0], img[1]), (W, H)
+    finally:
+        V.vdi_destroy(vdi)
