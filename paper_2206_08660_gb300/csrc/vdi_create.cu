@@ -97,16 +97,18 @@ __global__ void convert_kernel(const float *__restrict__ rgba, const float *__re
 // A supersegment [f, b] counts in slab k when f < edge[k+1] and b > edge[k]; a
 // zero-length one (f == b) counts in the slab with edge[k] <= f < edge[k+1].
 // With edges in order both conditions are monotone in k, so its slabs are one
-// run: a binary search finds its start, and it counts as +1 there and -1 after
-// its end (prefix sums give the counts; exact, no global atomics).
+// run, counted as +1 where it starts and -1 after its end (prefix sums give the
+// counts; exact, no global atomics); a list's supersegments are in order too, so
+// a run is looked for from the last one's end on.
 //
-// What bounds it: the depth records of the lists that hold anything.  A block
-// takes a row of kGridCols cells (its counts of a slab are one 32-byte run),
-// reads the ranges first and gathers the lists that are not empty; only their
-// slot pairs are read.  Each counter exists kGridCopies times, by lane, since
+// What bounds it: issue and the depth records of the lists that hold anything.
+// A block takes a row of kGridCols cells (its counts of a slab are one 32-byte
+// run), reads the ranges first and gathers the lists that are not empty; a
+// thread then walks one list up to its last supersegment, the next pair
+// requested ahead.  Each counter exists kGridCopies times, by lane, since
 // neighbouring lists count in the same slabs.
-// 1920 x 1080 lists of 20 slots (78% of them empty), ranges of 4 x 4 lists
-// included: one block per cell over every slot with a test per slab 136 us.
+// 1920 x 1080 lists of 20 slots (78% of them empty), block ranges included: one
+// block per cell over every slot with a test per slab 136 us, 50 us.
 constexpr int kGridCols = 8, kGridCopies = 8, kGridChunk = 512;
 
 __global__ void __launch_bounds__(256) grid_kernel(const DevVdi v, uint32_t *__restrict__ grid, float2 *__restrict__ brange) {
@@ -149,44 +151,40 @@ __global__ void __launch_bounds__(256) grid_kernel(const DevVdi v, uint32_t *__r
         __syncthreads();
         const int n = n_ids;
         any |= n > 0;
-        for (int it = t; it < n * npairs; it += blockDim.x) {
-            const int k = it / n;
-            const unsigned id = ids[it - k * n];
-            const int x = id & 0xffffu, y = id >> 16, col = x / T;
-            const float4 d = v.depth[(size_t)k * v.nl + (size_t)(y0 + y) * v.w + x0 + x];
-            const float fs[2] = {d.x, d.z}, bs[2] = {d.y, d.w};
+        for (int i = t; i < n; i += blockDim.x) {
+            const unsigned id = ids[i];
+            const int x = id & 0xffffu, y = id >> 16;
+            int *count = &cnt[x / T][t & (kGridCopies - 1)];  // of slab z: count[z * kGridCols * kGridCopies]
+            const float4 *rec = v.depth + (size_t)(y0 + y) * v.w + x0 + x;
+            float4 next = *rec;
+            int z = 0;  // no supersegment still to come lies in an earlier slab
+            for (int k = 0; k < npairs; ++k) {
+                const float4 d = next;
+                if (!isfinite(d.x)) break;
+                if (k + 1 < npairs) next = rec[(size_t)(k + 1) * v.nl];
+                const float fs[2] = {d.x, d.z}, bs[2] = {d.y, d.w};
 #pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                const float f = fs[s], b = bs[s];
-                if (!isfinite(f)) continue;
-                if (!ordered) {
-                    for (int z = 0; z < nz; ++z) {
-                        const bool hit = (f == b) ? (edges[z] <= f && f < edges[z + 1]) : (f < edges[z + 1] && b > edges[z]);
-                        if (hit) {
-                            atomicAdd(&cnt[z * kGridCols + col][t & (kGridCopies - 1)], 1);
-                            atomicAdd(&cnt[(z + 1) * kGridCols + col][t & (kGridCopies - 1)], -1);
+                for (int s = 0; s < 2; ++s) {
+                    const float f = fs[s], b = bs[s];
+                    if (!isfinite(f)) break;
+                    if (!ordered) {
+                        for (int q = 0; q < nz; ++q) {
+                            const bool hit = (f == b) ? (edges[q] <= f && f < edges[q + 1]) : (f < edges[q + 1] && b > edges[q]);
+                            if (hit) {
+                                atomicAdd(count + q * kGridCols * kGridCopies, 1);
+                                atomicAdd(count + (q + 1) * kGridCols * kGridCopies, -1);
+                            }
                         }
+                        continue;
                     }
-                    continue;
-                }
-                int lo = 0, hi = nz;  // first slab with f < edge[k+1]
-                while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
-                    if (f < edges[mid + 1])
-                        hi = mid;
-                    else
-                        lo = mid + 1;
-                }
-                int end = lo;  // first slab from there that fails the other condition
-                hi = nz;
-                while (end < hi) {
-                    const bool in = f == b ? edges[end] <= f : b > edges[end];
-                    if (!in) break;
-                    ++end;
-                }
-                if (end > lo) {
-                    atomicAdd(&cnt[lo * kGridCols + col][t & (kGridCopies - 1)], 1);
-                    atomicAdd(&cnt[end * kGridCols + col][t & (kGridCopies - 1)], -1);
+                    while (z < nz && !(f < edges[z + 1])) ++z;
+                    int end = z;
+                    while (end < nz && (f == b ? edges[end] <= f : b > edges[end])) ++end;
+                    if (end > z) {
+                        atomicAdd(count + z * kGridCols * kGridCopies, 1);
+                        atomicAdd(count + end * kGridCols * kGridCopies, -1);
+                        z = end - 1;
+                    }
                 }
             }
         }
