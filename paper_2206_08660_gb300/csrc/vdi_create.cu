@@ -32,7 +32,8 @@ __device__ __forceinline__ unsigned pack_half2(float a, float b) {
 // pair of all of them at a time: the input of a list is contiguous, so the
 // block's warps share its cache lines, and the stores are list-fastest.  (With
 // a block per slot pair every line of the input came from DRAM two to three
-// times: 201 us for 1366 x 767 lists of up to 15 slots, FP16 colour.)
+// times: 1366 x 767 lists of up to 15 slots, FP16 colour, 201 us against 100 us,
+// 69% of DRAM's peak.)
 // The list ranges are written on the way (front of the first, back of the last).
 template <int FMT>
 __global__ void convert_kernel(const float *__restrict__ rgba, const float *__restrict__ depth,
@@ -108,7 +109,7 @@ __global__ void convert_kernel(const float *__restrict__ rgba, const float *__re
 // requested ahead.  Each counter exists kGridCopies times, by lane, since
 // neighbouring lists count in the same slabs.
 // 1920 x 1080 lists of 20 slots (78% of them empty), block ranges included: one
-// block per cell over every slot with a test per slab 136 us, 50 us.
+// block per cell over every slot with a test per slab 136 us, this 50 us.
 constexpr int kGridCols = 8, kGridCopies = 8, kGridChunk = 512;
 
 __global__ void __launch_bounds__(256) grid_kernel(const DevVdi v, uint32_t *__restrict__ grid, float2 *__restrict__ brange) {
