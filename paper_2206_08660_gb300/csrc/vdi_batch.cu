@@ -30,7 +30,9 @@
 namespace vdi {
 
 constexpr int kMaxBatchReq = VDI_BATCH_MAX_REQUESTS;
-constexpr int kBatchLanes = 4;  // lanes per ray of a preview request
+constexpr int kBatchWarps = 4;                               // warps of a preview block
+constexpr int kBatchRays = 16;                                // preview rays per warp
+constexpr int kBatchCols = kBatchWarps * kBatchRays / 4;       // a block's tile: kBatchCols x 4 rays
 constexpr int kMaxBatchVdi = VDI_BATCH_MAX_VDIS;
 
 struct BatchReq {
@@ -42,9 +44,8 @@ struct BatchReq {
     int tile_base;   // first tile of this request in the queue
 };
 
-// Two tile queues: exact requests (32 x 8 tiles, one lane per ray) and
-// ray-subsampled previews (32 x (8 / kBatchLanes) tiles, kBatchLanes lanes per
-// ray), each pulled by its own persistent kernel from its own counter.  A
+// Two tile queues: exact requests (32 x 8 tiles) and ray-subsampled previews
+// (kBatchCols x 4 tiles), each pulled by its own persistent kernel from its own counter.  A
 // request's tile_base counts within its queue; ex_idx / pv_idx list the
 // requests of each queue in queue order.
 struct BatchParams {
@@ -128,25 +129,30 @@ __global__ void __launch_bounds__(256, 4) batch_render_kernel(const BatchParams 
     }
 }
 
-// Ray-subsampled previews: kBatchLanes lanes per ray (the same image as the
-// single-view kernels' lane counts).
-__global__ void __launch_bounds__(256, 3) batch_preview_kernel(const BatchParams P) {
-    constexpr int rows = 8 / kBatchLanes;
-    const int g = (int)threadIdx.x / kBatchLanes;
+// Ray-subsampled previews, kBatchRays rays per warp (the same image as the
+// single-view kernels' counts).
+__global__ void __launch_bounds__(32 * kBatchWarps, 7) batch_preview_kernel(const BatchParams P) {
+    __shared__ PreviewWarp<kBatchRays> warps[kBatchWarps];
+    __shared__ float edges[kMaxNz + 1];
+    const int warp = threadIdx.x >> 5;
     for (;;) {
         int r;
         const int tile = next_tile(P, P.pcounter, P.pv_idx, P.n_pv, P.total_ptiles, r);
         if (tile >= P.total_ptiles) return;
         const BatchReq &q = P.reqs[r];
         const DevVdi &v = P.vdis[q.vdi];
+        for (int k = threadIdx.x; k <= v.nz; k += blockDim.x) edges[k] = v.edges[k];
+        __syncthreads();  // (next_tile's first barrier keeps them until every warp is done)
         const int local = tile - q.tile_base;
-        const int px = (local % q.tiles_x) * 32 + (g & 31), py = (local / q.tiles_x) * rows + (g >> 5);
-        const bool inside = px < q.c.W && py < q.c.H;
+        int lx, ly;
+        preview_offset(warp * kBatchRays, lx, ly);
+        const int px = (local % q.tiles_x) * kBatchCols + lx, py = (local / q.tiles_x) * 4 + ly;
+        const bool inside = (threadIdx.x & 31) < kBatchRays && px < q.c.W && py < q.c.H;
         Ray ray = {};
         const bool active = inside && setup_ray<false>(q.c, px, py, v.w, v.h, ray);
-        const Accum acc = (v.fmt == 0) ? march_preview_lanes<0, kPreviewProbe, kBatchLanes>(v, q.c, ray, active)
-                                       : march_preview_lanes<1, kPreviewProbe, kBatchLanes>(v, q.c, ray, active);
-        if (inside && (threadIdx.x & (kBatchLanes - 1)) == 0) store_px(q.out, q.out_fmt, (size_t)py * q.c.W + px, acc);
+        const Accum acc = (v.fmt == 0) ? march_preview<0, kPreviewProbe, kBatchRays>(v, edges, q.c, warps[warp], ray, active)
+                                       : march_preview<1, kPreviewProbe, kBatchRays>(v, edges, q.c, warps[warp], ray, active);
+        if (inside) store_px(q.out, q.out_fmt, (size_t)py * q.c.W + px, acc);
     }
 }
 
@@ -239,9 +245,10 @@ static vdi_status plan_batch(vdi_ctx *ctx, const vdi_request *reqs, int n, Batch
         }
         q.vdi = vi;
         q.tiles_x = div_up(Wr, 32);
-        if (r.d_r > 1) {  // preview queue: 32 x (8 / kBatchLanes) tiles
+        if (r.d_r > 1) {  // preview queue: kBatchCols x 4 tiles
             q.tile_base = ptiles;
-            ptiles += q.tiles_x * div_up(Hr, 8 / kBatchLanes);
+            q.tiles_x = div_up(Wr, kBatchCols);
+            ptiles += q.tiles_x * div_up(Hr, 4);
             pl.bp->pv_idx[pl.bp->n_pv++] = (unsigned char)i;
         } else {  // exact queue: 32 x 8 tiles
             q.tile_base = tiles;
@@ -299,7 +306,7 @@ static int exact_grid(vdi_ctx *ctx, const BatchPlan &pl, int ws, int bps) {
 
 static int preview_grid(vdi_ctx *ctx, const BatchPlan &pl) {
     int occ = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void *)batch_preview_kernel, 256, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void *)batch_preview_kernel, 32 * kBatchWarps, 0);
     return std::min(std::max(1, occ) * ctx->sm_count, std::max(1, pl.bp->total_ptiles));
 }
 
@@ -310,7 +317,7 @@ static cudaError_t enqueue_plain(vdi_ctx *ctx, BatchPlan &pl, int ws, int bps, c
     if (pl.bp->n_ex) e = cudaLaunchKernel(render_fn(ws), dim3(exact_grid(ctx, pl, ws, bps)), dim3(256), args, 0, st);
     if (e != cudaSuccess) return e;
     if (pl.bp->n_pv)
-        e = cudaLaunchKernel((const void *)batch_preview_kernel, dim3(preview_grid(ctx, pl)), dim3(256), args, 0, st);
+        e = cudaLaunchKernel((const void *)batch_preview_kernel, dim3(preview_grid(ctx, pl)), dim3(32 * kBatchWarps), args, 0, st);
     if (e != cudaSuccess || pl.up->n == 0) return e;
     void *uargs[] = {pl.up};
     return cudaLaunchKernel((const void *)batch_upsample_kernel, dim3(pl.up->total_tiles), dim3(256), uargs, 0, st);
@@ -369,11 +376,11 @@ static std::string tune_key(const vdi_request *reqs, int n) {
     return k;
 }
 
-static cudaKernelNodeParams kernel_node(const void *fn, int grid, void **args) {
+static cudaKernelNodeParams kernel_node(const void *fn, int grid, int threads, void **args) {
     cudaKernelNodeParams kp{};
     kp.func = const_cast<void *>(fn);
     kp.gridDim = dim3(grid);
-    kp.blockDim = dim3(256);
+    kp.blockDim = dim3(threads);
     kp.kernelParams = args;
     return kp;
 }
@@ -407,17 +414,17 @@ static vdi_status enqueue_graph(vdi_ctx *ctx, const vdi_request *reqs, int n, Ba
         e = cudaGraphCreate(&ge.graph, 0);
         if (e == cudaSuccess) e = cudaGraphAddMemsetNode(&ms, ge.graph, nullptr, 0, &mp);
         if (e == cudaSuccess && pl.bp->n_ex) {
-            const cudaKernelNodeParams kp = kernel_node(render_fn(ws), ge.grid, args);
+            const cudaKernelNodeParams kp = kernel_node(render_fn(ws), ge.grid, 256, args);
             e = cudaGraphAddKernelNode(&ge.render_node, ge.graph, &ms, 1, &kp);
             renders.push_back(ge.render_node);
         }
         if (e == cudaSuccess && pl.bp->n_pv) {
-            const cudaKernelNodeParams kp = kernel_node((const void *)batch_preview_kernel, ge.pgrid, args);
+            const cudaKernelNodeParams kp = kernel_node((const void *)batch_preview_kernel, ge.pgrid, 32 * kBatchWarps, args);
             e = cudaGraphAddKernelNode(&ge.preview_node, ge.graph, &ms, 1, &kp);
             renders.push_back(ge.preview_node);
         }
         if (e == cudaSuccess && pl.up->n) {
-            const cudaKernelNodeParams kp = kernel_node((const void *)batch_upsample_kernel, pl.up->total_tiles, uargs);
+            const cudaKernelNodeParams kp = kernel_node((const void *)batch_upsample_kernel, pl.up->total_tiles, 256, uargs);
             e = cudaGraphAddKernelNode(&ge.up_node, ge.graph, renders.data(), renders.size(), &kp);
         }
         if (e == cudaSuccess) e = cudaGraphInstantiate(&ge.exec, ge.graph, 0);
@@ -431,15 +438,15 @@ static vdi_status enqueue_graph(vdi_ctx *ctx, const vdi_request *reqs, int n, Ba
         GraphEntry &ge = it->second;
         bind_scratch(pl, (char *)ge.scratch);
         if (ge.render_node) {
-            const cudaKernelNodeParams kp = kernel_node(render_fn(ws), ge.grid, args);
+            const cudaKernelNodeParams kp = kernel_node(render_fn(ws), ge.grid, 256, args);
             e = cudaGraphExecKernelNodeSetParams(ge.exec, ge.render_node, &kp);
         }
         if (e == cudaSuccess && ge.preview_node) {
-            const cudaKernelNodeParams kp = kernel_node((const void *)batch_preview_kernel, ge.pgrid, args);
+            const cudaKernelNodeParams kp = kernel_node((const void *)batch_preview_kernel, ge.pgrid, 32 * kBatchWarps, args);
             e = cudaGraphExecKernelNodeSetParams(ge.exec, ge.preview_node, &kp);
         }
         if (e == cudaSuccess && ge.up_node) {
-            const cudaKernelNodeParams kp = kernel_node((const void *)batch_upsample_kernel, pl.up->total_tiles, uargs);
+            const cudaKernelNodeParams kp = kernel_node((const void *)batch_upsample_kernel, pl.up->total_tiles, 256, uargs);
             e = cudaGraphExecKernelNodeSetParams(ge.exec, ge.up_node, &kp);
         }
         if (e != cudaSuccess) return cuda_fail(e, "graph update");

@@ -1,18 +1,25 @@
-// vdi_preview.cuh -- the ray-subsampled preview of Section 4.4 with several
-// lanes of a warp per ray.
+// vdi_preview.cuh -- the ray-subsampled preview of Section 4.4.
 //
 // A preview ray's samples are independent of one another once their positions
 // are known: each takes the supersegment that contains it, with opacity for
-// the sample spacing (Eq. 2).  Compositing is associative, so a ray's grid
-// cells can be composited in parallel and the partial results merged in
-// order.  The ray walks the count grid in rounds of kRoundCells cells; in a
-// round, each of the L lanes serving the ray composites kRoundCells / L
-// consecutive cells into a partial result, and the lanes merge the partials
-// with warp shuffles in a fixed balanced tree over the round's cells (so the
-// image does not depend on L).  Early termination is checked once per round.
-// Launches with few rays (a preview at a high D_I or D_R fills less than a
-// wave of the GPU with one lane per ray) run with more lanes per ray, which
-// cuts the chain of dependent loads each lane waits for.
+// the sample spacing (Eq. 2).  Compositing is associative, so the cells of the
+// count grid that a ray crosses can be composited apart and merged in order.
+//
+// A warp serves R rays, each walked by one lane in rounds of kRoundCells
+// cells.  Cells that hold something go to the warp's queue in shared memory,
+// and the warp takes 32 of them at a time, one per lane, whichever rays they
+// belong to; each composites to a partial result in shared memory, and a
+// round's partials are merged in a fixed balanced tree (so the image does not
+// depend on R).  Early termination is checked once per round.
+//
+// What bounds it: the latency of dependent gathers (count, list range and
+// depth pair, colour) and issue.  Walking a ray on every lane that serves it
+// cost half the instructions, and empty cells idled the lanes; with the queue
+// a step is taken once and the sampling lanes are full.  Launches with few
+// rays run with fewer rays per warp, which keeps more warps in flight.
+// GB300, whole previews of 1920 x 1080 lists (20 slots, FP16 colour) at 30
+// degrees: 960 x 540 rays 150 -> 119 us, 480 x 270 rays 68 -> 61 us, 1920 x 1080
+// rays 292 -> 254 us.
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
@@ -24,7 +31,8 @@
 namespace vdi {
 
 constexpr int kRoundCells = 8;    // grid cells per compositing round
-constexpr int kPreviewProbe = 2;  // depth records a preview sample requests at once
+constexpr int kPreviewProbe = 2;  // depth records a preview sample's scan requests at once
+constexpr int kPreviewWarps = 4;  // warps per block
 
 // a in front of b
 __device__ __forceinline__ Accum over(const Accum &a, const Accum &b) {
@@ -36,194 +44,290 @@ __device__ __forceinline__ Accum over(const Accum &a, const Accum &b) {
     return o;
 }
 
-// One grid cell of a ray: linear cell index, its footprint in lists, and the
-// ray's NDC line parameter range inside it (sb <= sa: nothing to sample).
+// One grid cell of a ray: linear cell index and the ray's NDC line parameter
+// range inside it (sb <= sa: nothing to sample).
 struct CellRec {
-    int cell, lists;
+    int cell;
     float sa, sb;
 };
 
 // The ray's walk over the cells of the count grid (T x T lists by slabs of
 // equal V_O view depth): Amanatides-Woo with boundary crossings computed
-// directly from integer offsets, as in the list walk.
+// directly from integer offsets, as in the list walk.  It ends at s_end, the
+// nearest of the ray's end and its crossings of the grid's far faces (the same
+// formula as every other crossing): a step along an axis is taken only while
+// the next boundary lies before that axis's face, so the indices need no
+// bounds tests.  The slab edges come from shared memory (every lane its own).
 struct CellWalk {
-    int cx, cy, cz, bx, by, ez, stx, sty;
-    float sx, sy, sz, s_in, idgx, idgy, idz;
-    bool ended;
+    int cell, ez;
+    float bx, by;  // next boundaries relative to the ray's integer origin
+    float sx, sy, sz, s_in, s_end;
+    float idgx, idgy, idz;  // their signs are the steps' directions
 };
 
-__device__ __forceinline__ void cell_walk_init(CellWalk &w, const DevVdi &v, const Ray &r, bool active) {
+__device__ __forceinline__ void cell_walk_init(CellWalk &w, const DevVdi &v, const float *edges, const Ray &r, bool active) {
     const int T = v.T;
-    w.cx = min(max(r.ox, 0) / T, v.gw - 1);
-    w.cy = min(max(r.oy, 0) / T, v.gh - 1);
-    w.stx = r.dgx > 0.f ? 1 : -1;
-    w.sty = r.dgy > 0.f ? 1 : -1;
+    const bool px = r.dgx > 0.f, py = r.dgy > 0.f, inc = r.dz >= 0.f;
+    const int col = min(max(r.ox, 0) / T, v.gw - 1), row = min(max(r.oy, 0) / T, v.gh - 1);
     w.idgx = rcp_fast(r.dgx);
     w.idgy = rcp_fast(r.dgy);
-    w.bx = (w.cx + (r.dgx > 0.f ? 1 : 0)) * T;
-    w.by = (w.cy + (r.dgy > 0.f ? 1 : 0)) * T;
-    w.sx = (r.dgx != 0.f) ? ((float)(w.bx - r.ox) - r.fx0) * w.idgx : INFINITY;
-    w.sy = (r.dgy != 0.f) ? ((float)(w.by - r.oy) - r.fy0) * w.idgy : INFINITY;
     w.idz = rcp_fast(r.dz);
-    const bool inc = r.dz >= 0.f;
-    w.cz = 0;
-    while (w.cz + 1 < v.nz && r.z0 >= v.edges[w.cz + 1]) ++w.cz;
-    w.ez = inc ? w.cz + 1 : w.cz;
-    w.sz = (r.dz != 0.f) ? (v.edges[w.ez] - r.z0) * w.idz : INFINITY;
+    w.bx = (float)((col + (px ? 1 : 0)) * T - r.ox);
+    w.by = (float)((row + (py ? 1 : 0)) * T - r.oy);
+    const bool mx = crosses(r.ox, r.fx0, w.idgx), my = crosses(r.oy, r.fy0, w.idgy);
+    const bool mz = fabsf(w.idz) < INFINITY && fabsf(r.z0) < INFINITY;
+    w.sx = mx ? (w.bx - r.fx0) * w.idgx : INFINITY;
+    w.sy = my ? (w.by - r.fy0) * w.idgy : INFINITY;
+    const float ex = mx ? ((float)((px ? v.gw * T : 0) - r.ox) - r.fx0) * w.idgx : INFINITY;
+    const float ey = my ? ((float)((py ? v.gh * T : 0) - r.oy) - r.fy0) * w.idgy : INFINITY;
+    int cz = 0;
+    while (cz + 1 < v.nz && r.z0 >= edges[cz + 1]) ++cz;
+    w.ez = inc ? cz + 1 : cz;
+    w.sz = mz ? (edges[w.ez] - r.z0) * w.idz : INFINITY;
+    const float ez = mz ? (edges[inc ? v.nz : 0] - r.z0) * w.idz : INFINITY;
+    w.cell = (cz * v.gh + row) * v.gw + col;
     w.s_in = 0.f;
-    w.ended = !active;
+    w.s_end = active ? fminf(fminf(fminf(ex, ey), ez), 1.f) : -1.f;
 }
 
 // The current cell, then a step to the next one.
-__device__ __forceinline__ CellRec cell_walk_next(CellWalk &w, const DevVdi &v, const Ray &r) {
+__device__ __forceinline__ CellRec cell_walk_next(CellWalk &w, const DevVdi &v, const float *edges, const Ray &r) {
     CellRec c;
-    const float s_out = fminf(fminf(fminf(w.sx, w.sy), w.sz), 1.f);
-    c.cell = (w.cz * v.gh + w.cy) * v.gw + w.cx;
-    c.lists = min(v.T, v.w - w.cx * v.T) * min(v.T, v.h - w.cy * v.T);
+    const float s_out = fminf(fminf(fminf(w.sx, w.sy), w.sz), w.s_end);
+    c.cell = w.cell;
     c.sa = w.s_in;
-    c.sb = w.ended ? w.s_in : s_out;
-    if (!w.ended) {
-        if (s_out >= 1.f) {
-            w.ended = true;
-        } else if (w.sx <= w.sy && w.sx <= w.sz) {
-            w.cx += w.stx;
-            if ((unsigned)w.cx >= (unsigned)v.gw) w.ended = true;
-            w.bx += w.stx * v.T;
-            w.sx = ((float)(w.bx - r.ox) - r.fx0) * w.idgx;
-        } else if (w.sy <= w.sz) {
-            w.cy += w.sty;
-            if ((unsigned)w.cy >= (unsigned)v.gh) w.ended = true;
-            w.by += w.sty * v.T;
-            w.sy = ((float)(w.by - r.oy) - r.fy0) * w.idgy;
-        } else {
-            const bool inc = r.dz >= 0.f;
-            w.cz += inc ? 1 : -1;
-            if ((unsigned)w.cz >= (unsigned)v.nz) w.ended = true;
-            w.ez += inc ? 1 : -1;
-            if (!w.ended) w.sz = (v.edges[w.ez] - r.z0) * w.idz;
+    c.sb = s_out;
+    if (s_out < w.s_end) {
+        const bool x = w.sx <= w.sy && w.sx <= w.sz, y = !x && w.sy <= w.sz;
+        if (x) {
+            w.cell += w.idgx > 0.f ? 1 : -1;
+            w.bx += copysignf((float)v.T, w.idgx);
+            w.sx = (w.bx - r.fx0) * w.idgx;
         }
-        w.s_in = fmaxf(w.s_in, s_out);
+        if (y) {
+            w.cell += w.idgy > 0.f ? v.gw : -v.gw;
+            w.by += copysignf((float)v.T, w.idgy);
+            w.sy = (w.by - r.fy0) * w.idgy;
+        }
+        if (!x && !y) {
+            w.cell += w.idz > 0.f ? v.gh * v.gw : -v.gh * v.gw;
+            w.ez += w.idz > 0.f ? 1 : -1;
+            w.sz = (edges[w.ez] - r.z0) * w.idz;
+        }
     }
+    w.s_in = fmaxf(w.s_in, s_out);
     return c;
 }
 
 // The samples of one cell (Section 4.4): in a cell holding cnt supersegments
 // over its lists, crossed over world length l_c, n = ceil((cnt / lists)
 // (l_c / slab depth extent) / D_R) samples at the midpoints of n equal
-// pieces; each finds the supersegment containing it with a probe of PW depth
-// records at a time (the first slot whose back reaches the sample's depth:
-// Algorithm 2's result) and is composited with opacity for the spacing.
-template <int FMT, int PW>
-__device__ __forceinline__ void preview_cell(const DevVdi &v, const ViewConsts &c, const Ray &r, const CellRec &rec,
-                                             Accum &part) {
-    if (!(rec.sb > rec.sa)) return;
-    const uint32_t cnt = __ldg(v.grid + rec.cell);
-    if (!cnt) return;
-    const float hw = 0.5f * (float)v.w, hh = 0.5f * (float)v.h;
+// pieces, u the ray's homogeneous parameter.
+struct CellSamples {
+    int n;
+    float ua, du, spacing;
+};
+
+// w: w0, w1, dw, lu of the ray
+__device__ __forceinline__ CellSamples cell_samples(const DevVdi &v, const ViewConsts &c, const float4 &w, const CellRec &rec,
+                                                    uint32_t cnt) {
+    CellSamples q;
     const float s_in = rec.sa, s_out = rec.sb;
-    const float ua = s_in * r.w0 * rcp_fast(fmaf(s_in, r.dw, r.w1));
-    const float ub = s_out * r.w0 * rcp_fast(fmaf(s_out, r.dw, r.w1));
-    const float lc = r.lu * (ub - ua);
-    const float want = ((float)cnt / (float)rec.lists) * lc * c.cell_scale;
-    // at least one sample per occupied cell; the cap only guards non-finite input
-    const int n = (want < 65536.f) ? max(1, (int)ceilf(want)) : 65536;
-    const float du = (ub - ua) / (float)n, spacing = lc / (float)n;
-    const int npairs = v.nsp >> 1;
-    for (int k = 0; k < n; ++k) {
-        const float uk = fmaf((float)k + 0.5f, du, ua);
-        const float hx = fmaf(uk, r.h1.x - r.h0.x, r.h0.x);
-        const float hy = fmaf(uk, r.h1.y - r.h0.y, r.h0.y);
-        const float hz = fmaf(uk, r.h1.z - r.h0.z, r.h0.z);
-        const float hwc = fmaf(uk, r.h1.w - r.h0.w, r.h0.w);
-        const float iw = rcp_fast(hwc);
-        const float nx = hx * iw, ny = hy * iw, nz = hz * iw;
-        const int jx = min(max((int)floorf((nx + 1.f) * hw), 0), v.w - 1);
-        const int jy = min(max((int)floorf((1.f - ny) * hh), 0), v.h - 1);
-        const int li = jy * v.w + jx;
-        const float2 rg = __ldg(v.range + li);
-        if (nz < rg.x || nz > rg.y) continue;  // outside every supersegment of the list
-        int j = v.nsp;
-        float fj = INFINITY;
-        for (int k0 = 0; k0 < npairs && j == v.nsp; k0 += PW) {
-            float4 d[PW];
-#pragma unroll
-            for (int i = 0; i < PW; ++i)
-                if (k0 + i < npairs) d[i] = ld_depth_pair(v, k0 + i, li);
-#pragma unroll
-            for (int i = PW - 1; i >= 0; --i)
-                if (k0 + i < npairs) {
-                    if (d[i].w >= nz) {
-                        j = 2 * (k0 + i) + 1;
-                        fj = d[i].z;
-                    }
-                    if (d[i].y >= nz) {
-                        j = 2 * (k0 + i);
-                        fj = d[i].x;
-                    }
-                }
-        }
-        if (j < v.nsp && fj <= nz) {
-            ColourCache<FMT> cc;
-            cc.k = -1;
-            add_piece(part, get_colour<FMT>(cc, v, li, j), spacing);
-        }
+    q.ua = s_in * w.x * rcp_fast(fmaf(s_in, w.z, w.y));
+    const float ub = s_out * w.x * rcp_fast(fmaf(s_out, w.z, w.y));
+    const float lc = w.w * (ub - q.ua);
+    int lists = v.T * v.T;
+    if (v.gw * v.T != v.w || v.gh * v.T != v.h) {  // cells at a ragged edge hold fewer
+        const int rows = rec.cell / v.gw;
+        lists = min(v.T, v.w - (rec.cell - rows * v.gw) * v.T) * min(v.T, v.h - rows % v.gh * v.T);
     }
+    // a power of two divides as exactly by its reciprocal
+    const float per_list = (lists & (lists - 1)) == 0 ? (float)cnt * __int_as_float((127 - (31 - __clz(lists))) << 23)
+                                                      : (float)cnt / (float)lists;
+    const float want = per_list * lc * c.cell_scale;
+    // at least one sample per occupied cell; the cap only guards non-finite input
+    q.n = (want < 65536.f) ? max(1, (int)ceilf(want)) : 65536;
+    q.du = ub - q.ua;
+    q.spacing = lc;
+    if (q.n > 1) {
+        q.du /= (float)q.n;
+        q.spacing /= (float)q.n;
+    }
+    return q;
 }
 
-// The preview of one ray served by L lanes (L in {2, 4, 8}: the lanes
-// threadIdx.x & ~(L - 1) .. + L - 1 of a warp; every lane of the warp must
-// call this, lanes without a ray with active = false).  Returns the ray's
-// composite in every lane of the group.
-template <int FMT, int PW, int L>
-__device__ __forceinline__ Accum march_preview_lanes(const DevVdi &v, const ViewConsts &c, const Ray &r,
-                                                     bool active) {
-    constexpr int G = kRoundCells / L;  // consecutive cells per lane and round
-    static_assert(L >= 2 && L <= kRoundCells && G * L == kRoundCells, "lanes per ray");
-    const unsigned full = 0xffffffffu;
-    const int sub = threadIdx.x & (L - 1);
+// One sample: the supersegment of its list that contains it (the first slot
+// whose back reaches its depth: Algorithm 2's result), composited with opacity
+// for the spacing.  The search starts at the pair where the ray's last sample
+// ended (`seed`: samples follow the depth, and neighbouring lists are alike),
+// requested together with the list's range: a sample inside the seed pair's
+// first supersegment needs no look before it, a pair further along is scanned
+// for, one before it is searched for from the front.
+template <int FMT, int PW>
+__device__ __forceinline__ void preview_sample(const DevVdi &v, const float4 &h0, const float4 &dh, const CellSamples &q,
+                                               int nth, int &seed, Accum &part) {
+    const float hw = 0.5f * (float)v.w, hh = 0.5f * (float)v.h;
+    const float uk = fmaf((float)nth + 0.5f, q.du, q.ua);
+    const float hx = fmaf(uk, dh.x, h0.x);
+    const float hy = fmaf(uk, dh.y, h0.y);
+    const float hz = fmaf(uk, dh.z, h0.z);
+    const float hwc = fmaf(uk, dh.w, h0.w);
+    const float iw = rcp_fast(hwc);
+    const float nx = hx * iw, ny = hy * iw, nz = hz * iw;
+    const int jx = min(max((int)floorf((nx + 1.f) * hw), 0), v.w - 1);
+    const int jy = min(max((int)floorf((1.f - ny) * hh), 0), v.h - 1);
+    const int li = jy * v.w + jx;
+    const float2 rg = __ldg(v.range + li);
+    const float4 ds = ld_depth_pair(v, seed, li);
+    if (nz < rg.x || nz > rg.y) return;  // outside every supersegment of the list
+    // slot pair k with record d holds the answer, or k = npairs: not found yet,
+    // every pair before k0 ends before the sample.  (The lanes' cases share
+    // their loads, so that they run together.)
+    const int npairs = v.nsp >> 1;
+    const bool reached = ds.w >= nz;
+    const int kp = reached ? seed - 1 : seed + 1;
+    int k = reached ? seed : npairs, k0 = npairs;
+    float4 d = ds;
+    if (!(reached && ds.x < nz) && (unsigned)kp < (unsigned)npairs) {
+        const float4 dp = ld_depth_pair(v, kp, li);
+        if (dp.w >= nz) {
+            k = kp;
+            d = dp;
+            if (reached && !(dp.x < nz) && kp > 0) {
+                k = npairs;
+                k0 = 0;
+            }
+        } else if (!reached) {
+            k0 = kp + 1;
+        }
+    }
+    for (; k0 < npairs && k == npairs; k0 += PW) {
+        float4 dd[PW];
+#pragma unroll
+        for (int i = 0; i < PW; ++i)
+            if (k0 + i < npairs) dd[i] = ld_depth_pair(v, k0 + i, li);
+#pragma unroll
+        for (int i = PW - 1; i >= 0; --i)
+            if (k0 + i < npairs && dd[i].w >= nz) {
+                k = k0 + i;
+                d = dd[i];
+            }
+    }
+    const int j = 2 * k + (d.y >= nz ? 0 : 1);
+    const float fj = d.y >= nz ? d.x : d.z;
+    if (k < npairs && fj <= nz) {
+        ColourCache<FMT> cc;
+        cc.k = -1;
+        add_piece(part, get_colour<FMT>(cc, v, li, j), q.spacing);
+    }
+    seed = min(k, npairs - 1);
+}
+
+constexpr int kWalkBatch = 4;                        // steps whose counts are requested together
+constexpr int kPreviewQueue = 32 + 32 * kWalkBatch;  // a batch adds to fewer than 32
+
+// A warp's shared memory: its rays, the queue of occupied cells, the partial results.
+template <int R>
+struct PreviewWarp {
+    float4 part[R][kRoundCells];  // of the round's occupied cells
+    float4 h0[R], dh[R];     // homogeneous clip coordinates of the ray's start, and to its end
+    float4 w[R];             // w0, w1, dw, lu of the ray
+    int seed[R];             // the slot pair where the ray's last sample ended
+    int4 queue[kPreviewQueue];  // sa, sb (bits), cell, supersegments there
+    int owner[kPreviewQueue];   // ray + 32 cell of the round
+};
+
+// the last n (at most 32) queued cells to their partial results
+template <int FMT, int PW, int R>
+__device__ __forceinline__ void preview_queue(const DevVdi &v, const ViewConsts &c, PreviewWarp<R> &S, int &qn, int n) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    if (lane < n) {
+        const int e = qn - n + lane, id = S.owner[e], ray = id & 31;
+        const float4 w = S.w[ray], h0 = S.h0[ray], dh = S.dh[ray];
+        const int4 u = S.queue[e];
+        const CellSamples q = cell_samples(v, c, w, {u.z, __int_as_float(u.x), __int_as_float(u.y)}, (uint32_t)u.w);
+        Accum part = {0.f, 0.f, 0.f, 1.f};
+        int seed = S.seed[ray];
+        for (int k = 0; k < q.n; ++k) preview_sample<FMT, PW>(v, h0, dh, q, k, seed, part);
+        S.seed[ray] = seed;  // any lane's: a seed only starts the search
+        S.part[ray][id >> 5] = make_float4(part.r, part.g, part.b, part.T);
+    }
+    qn -= n;
+    __syncwarp();
+}
+
+// The previews of the R rays of a warp's first R lanes (R in {8, 16, 32}; every
+// lane of the warp must call this, lanes without a ray with active = false).
+// edges: the VDI's slab edges in shared memory.
+template <int FMT, int PW, int R>
+__device__ __forceinline__ Accum march_preview(const DevVdi &v, const float *edges, const ViewConsts &c, PreviewWarp<R> &S,
+                                               const Ray &r, bool active) {
+    constexpr int B = kWalkBatch;
+    static_assert(kRoundCells % B == 0, "whole batches per round");
+    const int lane = threadIdx.x & 31;
+    if (lane < R) {
+        S.h0[lane] = r.h0;
+        S.dh[lane] = make_float4(r.h1.x - r.h0.x, r.h1.y - r.h0.y, r.h1.z - r.h0.z, r.h1.w - r.h0.w);
+        S.w[lane] = make_float4(r.w0, r.w1, r.dw, r.lu);
+        S.seed[lane] = 0;
+    }
     CellWalk w;
-    cell_walk_init(w, v, r, active);
+    cell_walk_init(w, v, edges, r, active);
     Accum acc = {0.f, 0.f, 0.f, 1.f};
     bool going = active;
     const int maxr = (v.gw + v.gh + v.nz + 3 + kRoundCells - 1) / kRoundCells + 1;
-    for (int round = 0; round < maxr && __any_sync(full, going); ++round) {
-        // every lane steps through the round's cells and keeps its own G
-        CellRec rec[G];
+    for (int round = 0; round < maxr && __any_sync(~0u, going); ++round) {
+        int qn = 0;
+        unsigned occupied = 0;  // this ray's cells of the round that were queued
+#pragma unroll 1
+        for (int i0 = 0; i0 < kRoundCells; i0 += B) {
+            CellRec rec[B];
+            uint32_t cnt[B];
 #pragma unroll
-        for (int i = 0; i < kRoundCells; ++i) {
-            const CellRec cur = cell_walk_next(w, v, r);
-            if (i / G == sub) rec[i % G] = cur;
+            for (int i = 0; i < B; ++i) {
+                rec[i] = cell_walk_next(w, v, edges, r);
+                cnt[i] = (going && rec[i].sb > rec[i].sa) ? __ldg(v.grid + rec[i].cell) : 0u;
+            }
+#pragma unroll
+            for (int i = 0; i < B; ++i) {
+                const unsigned m = __ballot_sync(~0u, cnt[i] != 0u);
+                if (cnt[i]) {
+                    const int e = qn + __popc(m & ((1u << lane) - 1u));
+                    S.queue[e] = make_int4(__float_as_int(rec[i].sa), __float_as_int(rec[i].sb), rec[i].cell, (int)cnt[i]);
+                    S.owner[e] = lane | (i0 + i) << 5;
+                    occupied |= 1u << (i0 + i);
+                }
+                qn += __popc(m);
+            }
+            while (qn >= (i0 + B < kRoundCells ? 32 : 1)) preview_queue<FMT, PW, R>(v, c, S, qn, min(qn, 32));
         }
-        Accum part[G];
+        if (occupied) {
+            Accum p[kRoundCells];
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
-            part[g] = {0.f, 0.f, 0.f, 1.f};
-            if (going) preview_cell<FMT, PW>(v, c, r, rec[g], part[g]);
+            for (int i = 0; i < kRoundCells; ++i) {
+                float4 x = make_float4(0.f, 0.f, 0.f, 1.f);
+                if (occupied >> i & 1u) x = S.part[lane][i];
+                p[i] = {x.x, x.y, x.z, x.w};
+            }
+#pragma unroll
+            for (int s = 1; s < kRoundCells; s <<= 1)
+#pragma unroll
+                for (int i = 0; i + s < kRoundCells; i += 2 * s) p[i] = over(p[i], p[i + s]);
+            acc = over(acc, p[0]);
         }
-        // the lane's cells, then the lanes, merged as one balanced tree over the round's cells
-#pragma unroll
-        for (int s = 1; s < G; s <<= 1)
-#pragma unroll
-            for (int g = 0; g + s < G; g += 2 * s) part[g] = over(part[g], part[g + s]);
-        Accum x = part[0];
-#pragma unroll
-        for (int off = 1; off < L; off <<= 1) {
-            Accum o;
-            o.r = __shfl_down_sync(full, x.r, off, L);
-            o.g = __shfl_down_sync(full, x.g, off, L);
-            o.b = __shfl_down_sync(full, x.b, off, L);
-            o.T = __shfl_down_sync(full, x.T, off, L);
-            if ((sub & (2 * off - 1)) == 0) x = over(x, o);
-        }
-        Accum round_total;
-        round_total.r = __shfl_sync(full, x.r, 0, L);
-        round_total.g = __shfl_sync(full, x.g, 0, L);
-        round_total.b = __shfl_sync(full, x.b, 0, L);
-        round_total.T = __shfl_sync(full, x.T, 0, L);
-        if (going) acc = over(acc, round_total);
-        if (acc.T <= kErtT || w.ended) going = false;
+        if (acc.T <= kErtT || w.s_in >= w.s_end) going = false;
+        __syncwarp();
     }
     return acc;
+}
+
+// The ray of a warp's lane within a 32 x 8 tile: rays in 8 x 4 patches, a warp
+// on R consecutive ones.  first: the warp's first ray of the tile's 256.
+__device__ __forceinline__ void preview_offset(int first, int &dx, int &dy) {
+    const int i = first + (int)(threadIdx.x & 31), patch = i >> 5;
+    dx = (patch & 3) * 8 + (i & 7);
+    dy = (patch >> 2) * 4 + ((i >> 3) & 3);
 }
 
 }  // namespace vdi

@@ -195,44 +195,52 @@ __global__ void __launch_bounds__(256, RenderOccupancy<5>::blocks)
     if (!ready) mbar_wait(&bar, 0);  // no copy into this block's shared memory may outlive it
 }
 
-// Ray-subsampled preview (Section 4.4) with L lanes per ray: the blocks of a
-// 32 x 8 tile meeting the box's pixel rectangle (L blocks per tile, 256 / L
-// rays each) come first, then the fill blocks of the tiles outside it.
-template <int FMT, int L>
-__global__ void __launch_bounds__(256, 4) preview_kernel(const ViewConsts c, const DevVdi v, void *out, int out_fmt) {
-    constexpr int ROWS = 8 / L;  // tile rows per block
-    const int nrect = c.tile_w * c.tile_h;
-    if ((int)blockIdx.x >= nrect * L) {
-        fill_tiles(c, out, out_fmt, nullptr, nullptr, (int)blockIdx.x - nrect * L);
+// Ray-subsampled preview (Section 4.4) with R rays per warp: the blocks of a
+// 32 x 8 tile meeting the box's pixel rectangle (4 R rays each) come first,
+// then the fill blocks of the tiles outside it.  Seven blocks per SM: six (no
+// spills) 5%, eight 15% slower for 960 x 540 rays.
+template <int FMT, int R>
+__global__ void __launch_bounds__(32 * kPreviewWarps, 7) preview_kernel(const ViewConsts c, const DevVdi v, void *out,
+                                                                             int out_fmt) {
+    constexpr int S = 256 / (kPreviewWarps * R);  // blocks per tile
+    __shared__ PreviewWarp<R> warps[kPreviewWarps];
+    __shared__ float edges[kMaxNz + 1];
+    const int nunits = c.tile_w * c.tile_h * S;
+    if ((int)blockIdx.x >= nunits) {
+        fill_tiles(c, out, out_fmt, nullptr, nullptr, (int)blockIdx.x - nunits);
         return;
     }
-    const int tile = (int)blockIdx.x / L, unit = (int)blockIdx.x - tile * L;
-    int tx, ty;
+    for (int k = threadIdx.x; k <= v.nz; k += blockDim.x) edges[k] = v.edges[k];
+    __syncthreads();
+    const int tile = (int)blockIdx.x / S, unit = (int)blockIdx.x - tile * S, warp = threadIdx.x >> 5;
+    int lx, ly, tx, ty;
+    preview_offset((unit * kPreviewWarps + warp) * R, lx, ly);
     tile_of_block(c, tile, tx, ty);
-    const int g = (int)threadIdx.x / L;  // this lane's ray within the block
-    const int px = tx * 32 + (g & 31), py = ty * 8 + unit * ROWS + (g >> 5);
-    const bool inside = px < c.W && py < c.H;
+    const int px = tx * 32 + lx, py = ty * 8 + ly;
+    const bool inside = (threadIdx.x & 31) < R && px < c.W && py < c.H;
     Ray r = {};
     const bool active = inside && setup_ray<false>(c, px, py, v.w, v.h, r);
-    const Accum acc = march_preview_lanes<FMT, kPreviewProbe, L>(v, c, r, active);
-    if (inside && (threadIdx.x & (L - 1)) == 0) store_px(out, out_fmt, (size_t)py * c.W + px, acc);
+    const Accum acc = march_preview<FMT, kPreviewProbe, R>(v, edges, c, warps[warp], r, active);
+    if (inside) store_px(out, out_fmt, (size_t)py * c.W + px, acc);
 }
 
-template <int FMT, int L>
-static cudaError_t launch_preview_l(const ViewConsts &c, const DevVdi &v, void *out, int out_fmt, cudaStream_t st) {
+template <int FMT, int R>
+static cudaError_t launch_preview_r(const ViewConsts &c, const DevVdi &v, void *out, int out_fmt, cudaStream_t st) {
     const int nrect = c.tile_w * c.tile_h, ntiles = div_up(c.W, 32) * div_up(c.H, 8);
-    preview_kernel<FMT, L><<<nrect * L + div_up(ntiles - nrect, kFillTiles), 256, 0, st>>>(c, v, out, out_fmt);
+    const int grid = nrect * (256 / (kPreviewWarps * R)) + div_up(ntiles - nrect, kFillTiles);
+    preview_kernel<FMT, R><<<grid, 32 * kPreviewWarps, 0, st>>>(c, v, out, out_fmt);
     return cudaGetLastError();
 }
 
-// lanes per preview ray: more for launches with few rays, whose time is the
-// longest ray's chain of dependent loads (the image is the same for any count)
+// rays per warp: fewer for launches with few rays, whose time is the longest
+// ray's chain of dependent loads (the image is the same for any count).
+// 480 x 270 rays: 8 per warp 61 us, 16 75 us; 640 x 360 50 and 58 us;
+// 960 x 540 16 per warp 6% faster than 8; 32 gain nothing at 1920 x 1080.
 template <int FMT>
 static cudaError_t launch_preview(const ViewConsts &c, const DevVdi &v, void *out, int out_fmt, cudaStream_t st) {
     const long long rays = (long long)c.W * c.H;
-    if (rays <= 300000) return launch_preview_l<FMT, 8>(c, v, out, out_fmt, st);
-    if (rays <= 1200000) return launch_preview_l<FMT, 4>(c, v, out, out_fmt, st);
-    return launch_preview_l<FMT, 2>(c, v, out, out_fmt, st);
+    if (rays <= 300000) return launch_preview_r<FMT, 8>(c, v, out, out_fmt, st);
+    return launch_preview_r<FMT, 16>(c, v, out, out_fmt, st);
 }
 
 // Instrumented exact render: marks the VDI words the algorithm reads.

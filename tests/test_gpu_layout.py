@@ -96,7 +96,7 @@ def test_walk_equals_the_searching_walk(V, ctx, w, h, ns, fmt):
 
 @pytest.mark.parametrize("w, h, ns, fmt", [(40, 24, 2, 1), (67, 41, 5, 0), (33, 65, 33, 1)])
 def test_preview_rays_per_warp(V, ctx, w, h, ns, fmt):
-    """Previews at the sizes where the rays per warp change (8, 16, 32 in a launch
+    """Previews at the sizes where the rays per warp change (8 or 16 in a launch
     of its own, 16 in a batch): the same image, bit for bit."""
     case = random_case(w, h, ns, seed=w)
     vdi = V.vdi_create(ctx, case.gpu_desc(V, fmt), case.vdi.rgba, case.vdi.depth, case.vdi.counts)
