@@ -234,11 +234,14 @@ static cudaError_t launch_preview_r(const ViewConsts &c, const DevVdi &v, void *
 
 // rays per warp: fewer for launches with few rays, whose time is the longest
 // ray's chain of dependent loads (the image is the same for any count).
-// 480 x 270 rays: 8 per warp 61 us, 16 75 us; 640 x 360 50 and 58 us;
-// 960 x 540 16 per warp 6% faster than 8; 32 gain nothing at 1920 x 1080.
+// After an L2 flush, 4 / 8 / 16 rays per warp: 256 x 144 rays 27 / 35 / 35 us,
+// 320 x 180 42 / 51 / 51, 480 x 270 71 / 69 / 76 (on changing inputs 4 is the
+// faster by 1%), 640 x 360 70 / 57 / 58, 960 x 540 176 / 134 / 122, 1920 x 1080
+// 551 / 344 / 254.
 template <int FMT>
 static cudaError_t launch_preview(const ViewConsts &c, const DevVdi &v, void *out, int out_fmt, cudaStream_t st) {
     const long long rays = (long long)c.W * c.H;
+    if (rays <= 160000) return launch_preview_r<FMT, 4>(c, v, out, out_fmt, st);
     if (rays <= 300000) return launch_preview_r<FMT, 8>(c, v, out, out_fmt, st);
     return launch_preview_r<FMT, 16>(c, v, out, out_fmt, st);
 }

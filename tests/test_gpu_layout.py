@@ -96,12 +96,12 @@ def test_walk_equals_the_searching_walk(V, ctx, w, h, ns, fmt):
 
 @pytest.mark.parametrize("w, h, ns, fmt", [(40, 24, 2, 1), (67, 41, 5, 0), (33, 65, 33, 1)])
 def test_preview_rays_per_warp(V, ctx, w, h, ns, fmt):
-    """Previews at the sizes where the rays per warp change (8 or 16 in a launch
+    """Previews at the sizes where the rays per warp change (4, 8 or 16 in a launch
     of its own, 16 in a batch): the same image, bit for bit."""
     case = random_case(w, h, ns, seed=w)
     vdi = V.vdi_create(ctx, case.gpu_desc(V, fmt), case.vdi.rgba, case.vdi.depth, case.vdi.counts)
     try:
-        for W, H in ((5, 3), (40, 30), (800, 600), (1601, 903)):
+        for W, H in ((5, 3), (40, 30), (500, 300), (800, 600), (1601, 903)):
             cn = S.orbit_camera(case.bmin, case.bmax, W / H, az_deg=30, el_deg=15)
             cam = V.camera(cn.view, cn.proj)
             img = [torch.zeros((H, W, 4), device="cuda") for _ in range(2)]
