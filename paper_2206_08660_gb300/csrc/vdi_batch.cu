@@ -2,7 +2,7 @@
 // launch, optionally replayed from a CUDA graph, plus the batch autotuner.
 //
 // Exact requests are cut into 32 x 8 pixel tiles, ray-subsampled previews into
-// 32 x 2 tiles; each kind forms one queue, drained by its own persistent grid
+// 16 x 4 tiles; each kind forms one queue, drained by its own persistent grid
 // (SM count x resident blocks per SM) pulling tiles from an atomic counter, so
 // requests of different resolutions, previews and VDIs share the GPU without a
 // launch per view.  Requests with image-space
@@ -101,19 +101,23 @@ __device__ __forceinline__ int next_tile(const BatchParams &P, unsigned *counter
     return t;
 }
 
-// Exact requests: the list walk of vdi_render, one lane per ray.
+// Exact requests: the list walk of vdi_render, one lane per ray.  Blocks of
+// four warps, each half a tile: a block waits for its slowest warp before it
+// takes the next half.
+constexpr int kExactThreads = 128, kExactUnits = 256 / kExactThreads;
+
 template <int WX>
-__global__ void __launch_bounds__(256, 4) batch_render_kernel(const BatchParams P) {
+__global__ void __launch_bounds__(kExactThreads, 1024 / kExactThreads) batch_render_kernel(const BatchParams P) {
     for (;;) {
         int r;
-        const int tile = next_tile(P, P.counter, P.ex_idx, P.n_ex, P.total_tiles, r);
-        if (tile >= P.total_tiles) return;  // uniform: every thread read the same tile
+        const int half = next_tile(P, P.counter, P.ex_idx, P.n_ex, P.total_tiles, r);
+        if (half >= P.total_tiles) return;  // uniform: every thread read the same one
         const BatchReq &q = P.reqs[r];
         const DevVdi &v = P.vdis[q.vdi];
-        const int local = tile - q.tile_base;
+        const int local = (half - q.tile_base) / kExactUnits, unit = (half - q.tile_base) % kExactUnits;
         const int tx0 = (local % q.tiles_x) * 32, ty0 = (local / q.tiles_x) * 8;
         int lx, ly;
-        tile_offset<WX>(lx, ly);
+        tile_offset<WX>(unit * kExactThreads + (int)threadIdx.x, lx, ly);
         const int px = tx0 + lx, py = ty0 + ly;
         if (px < q.c.W && py < q.c.H) {
             Accum acc = {0.f, 0.f, 0.f, 1.f};
@@ -250,9 +254,9 @@ static vdi_status plan_batch(vdi_ctx *ctx, const vdi_request *reqs, int n, Batch
             q.tiles_x = div_up(Wr, kBatchCols);
             ptiles += q.tiles_x * div_up(Hr, 4);
             pl.bp->pv_idx[pl.bp->n_pv++] = (unsigned char)i;
-        } else {  // exact queue: 32 x 8 tiles
+        } else {  // exact queue: 32 x 8 tiles in kExactUnits parts
             q.tile_base = tiles;
-            tiles += q.tiles_x * div_up(Hr, 8);
+            tiles += q.tiles_x * div_up(Hr, 8) * kExactUnits;
             pl.bp->ex_idx[pl.bp->n_ex++] = (unsigned char)i;
         }
         pl.final_out[i] = r.out;
@@ -295,12 +299,12 @@ static void bind_scratch(BatchPlan &pl, char *scratch) {
         }
 }
 
-// persistent grid of the exact kernel: resident blocks per SM (capped at bps
+// persistent grid of the exact kernel: resident blocks per SM (capped at bps of 256 threads
 // when bps > 0) times the SM count, no more blocks than tiles
 static int exact_grid(vdi_ctx *ctx, const BatchPlan &pl, int ws, int bps) {
     int occ = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, render_fn(ws), 256, 0);
-    if (bps > 0) occ = std::min(occ, bps);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, render_fn(ws), kExactThreads, 0);
+    if (bps > 0) occ = std::min<long long>(occ, (long long)bps * kExactUnits);
     return std::min(std::max(1, occ) * ctx->sm_count, std::max(1, pl.bp->total_tiles));
 }
 
@@ -314,7 +318,7 @@ static cudaError_t enqueue_plain(vdi_ctx *ctx, BatchPlan &pl, int ws, int bps, c
     cudaError_t e = cudaMemsetAsync(pl.bp->counter, 0, 2 * sizeof(unsigned), st);
     if (e != cudaSuccess) return e;
     void *args[] = {pl.bp};
-    if (pl.bp->n_ex) e = cudaLaunchKernel(render_fn(ws), dim3(exact_grid(ctx, pl, ws, bps)), dim3(256), args, 0, st);
+    if (pl.bp->n_ex) e = cudaLaunchKernel(render_fn(ws), dim3(exact_grid(ctx, pl, ws, bps)), dim3(kExactThreads), args, 0, st);
     if (e != cudaSuccess) return e;
     if (pl.bp->n_pv)
         e = cudaLaunchKernel((const void *)batch_preview_kernel, dim3(preview_grid(ctx, pl)), dim3(32 * kBatchWarps), args, 0, st);
@@ -414,7 +418,7 @@ static vdi_status enqueue_graph(vdi_ctx *ctx, const vdi_request *reqs, int n, Ba
         e = cudaGraphCreate(&ge.graph, 0);
         if (e == cudaSuccess) e = cudaGraphAddMemsetNode(&ms, ge.graph, nullptr, 0, &mp);
         if (e == cudaSuccess && pl.bp->n_ex) {
-            const cudaKernelNodeParams kp = kernel_node(render_fn(ws), ge.grid, 256, args);
+            const cudaKernelNodeParams kp = kernel_node(render_fn(ws), ge.grid, kExactThreads, args);
             e = cudaGraphAddKernelNode(&ge.render_node, ge.graph, &ms, 1, &kp);
             renders.push_back(ge.render_node);
         }
@@ -438,7 +442,7 @@ static vdi_status enqueue_graph(vdi_ctx *ctx, const vdi_request *reqs, int n, Ba
         GraphEntry &ge = it->second;
         bind_scratch(pl, (char *)ge.scratch);
         if (ge.render_node) {
-            const cudaKernelNodeParams kp = kernel_node(render_fn(ws), ge.grid, 256, args);
+            const cudaKernelNodeParams kp = kernel_node(render_fn(ws), ge.grid, kExactThreads, args);
             e = cudaGraphExecKernelNodeSetParams(ge.exec, ge.render_node, &kp);
         }
         if (e == cudaSuccess && ge.preview_node) {
