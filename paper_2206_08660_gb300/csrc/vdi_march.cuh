@@ -442,9 +442,9 @@ __device__ __forceinline__ bool crosses(int o, float f0, float idg) {
 //    the binary search.
 //  * The slots of a pair are walked without index arithmetic, and the next pair
 //    is requested only when the list goes on (back before the range's end).
-// GB300, frames back to back: 1080p at 20 degrees of 1920 x 1080 lists (20
-// slots, FP16 colour) 327 -> 259 us, 720p at 15 degrees (256^3 noise, FP32
-// colour) 225 -> 150 us, 128 x 128 24.6 -> 18.8 us.  Requesting the next list's
+// GB300, whole calls on changing inputs: 1080p at 20 degrees of 1920 x 1080
+// lists (20 slots, FP16 colour) 324 -> 239 us, 720p at 15 degrees (256^3 noise,
+// FP32 colour) 237 -> 196 us, 128 x 128 26.7 -> 21.5 us.  Requesting the next list's
 // seed pair a step ahead, or the seed before the range test, gains nothing.
 // DIR: the sign of the ray's depth slope.
 template <int FMT, int DIR>
