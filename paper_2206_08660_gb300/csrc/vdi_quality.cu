@@ -68,10 +68,11 @@ __device__ __forceinline__ float2 fma_x2(float2 a, float2 b, float2 c) {
 
 // x / y, y a compile-time constant: the correctly rounded quotient from its
 // reciprocal (Markstein, IBM J. Res. Dev. 34, 1990) away from underflow, where
-// the windows' constants C1 and C2 swallow the difference
+// the windows' constants C1 and C2 swallow the difference.  An infinite x (a
+// variance that overflowed) has no residual: it stays infinite.
 __device__ __forceinline__ float div_const(float x, float y) {
     const float z = 1.f / y, q = x * z;
-    return fmaf(fmaf(-q, y, x), z, q);
+    return fabsf(q) < INFINITY ? fmaf(fmaf(-q, y, x), z, q) : q;
 }
 
 // A float as a double without the FP64 pipe's conversion

@@ -1,0 +1,69 @@
+"""Inputs at the edges of what the calls accept: pixels that overflow FP32
+variances, infinite and NaN pixels, sums whose terms differ by many orders of
+magnitude, eyes so far away that FP32 positions miss the box."""
+import math
+
+import numpy as np
+import pytest
+
+import vdi_synth as S
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def V():
+    import paper_2206_08660_gb300 as V
+
+    V.load()
+    return V
+
+
+@pytest.fixture(scope="module")
+def ctx(V):
+    c = V.vdi_ctx_create(0)
+    yield c
+    V.vdi_ctx_destroy(c)
+
+
+@pytest.mark.parametrize("W,H", [(7, 7), (9, 12), (70, 45)])
+@pytest.mark.parametrize("which", [0, 1, 2])
+def test_ssim_where_a_variance_overflows(V, W, H, which):
+    """Finite pixels of alternating sign whose sum of squares leaves FP32 while
+    the means and the covariance do not: SSIM is about 0 there, not NaN."""
+    from oracle import quality as Q
+
+    rng = np.random.default_rng(W)
+    sign = 1.0 - 2.0 * (np.add.outer(np.arange(H), np.arange(W)) % 2)
+    huge = np.repeat((3e19 * sign)[..., None], 4, axis=2).astype(np.float32)
+    plain = rng.uniform(0, 1, (H, W, 4)).astype(np.float32)
+    a, b = [(huge, plain), (plain, huge), (huge, 0.5 * huge)][which]
+    ssim, _ = V.vdi_image_quality(torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda())
+    if which < 2:
+        assert abs(Q.ssim(a, b)) < 1e-6 and abs(ssim) < 2e-6
+    else:  # the covariance overflows too: inf / inf
+        assert math.isnan(ssim)
+
+
+@pytest.mark.parametrize("fmt", [0, 1])
+@pytest.mark.parametrize("at", [(0, 0), (3, 5), (18, 37), (44, 69)])
+@pytest.mark.parametrize("pa, pb, psnr", [(float("nan"), 0.5, "inf"), (float("inf"), 0.5, "-inf"), (0.5, float("-inf"), "-inf"),
+                                          (float("inf"), float("inf"), "inf")])
+def test_quality_of_infinite_and_nan_pixels(V, fmt, at, pa, pb, psnr):
+    """SSIM is NaN; PSNR is -inf at an infinite error and +inf where the error is
+    NaN (the call's value for a mean squared error that is not above 0)."""
+    W, H = 70, 45
+    rng = np.random.default_rng(1)
+    img = [rng.uniform(0, 1, (H, W, 4)).astype(np.float32) for _ in range(2)]
+    for k, p in enumerate((pa, pb)):
+        img[k][at[0], at[1], 1] = p
+    dt = torch.float32 if fmt == 0 else torch.float16
+    ssim, got = V.vdi_image_quality(*[torch.from_numpy(i).to(dt).cuda() for i in img], fmt)
+    assert math.isnan(ssim)
+    assert got == float(psnr)
+    for k in range(2):  # the fourth channel is not measured
+        img[k][at[0], at[1], 1] = 0.5
+        img[k][at[0], at[1], 3] = (pa, pb)[k]
+    ssim, got = V.vdi_image_quality(*[torch.from_numpy(i).to(dt).cuda() for i in img], fmt)
+    assert math.isfinite(ssim) and math.isfinite(got)
