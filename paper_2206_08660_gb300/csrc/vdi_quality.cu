@@ -17,11 +17,14 @@
 // instruction; every window still adds its pixels row by row, left to right.
 // A block's 32 x 16 windows read a 38 x 22 pixel footprint staged in shared
 // memory.  FP64 (a narrow pipe: a third of the time when every difference was
-// converted) is left to one multiply-add per channel of a pixel that differs
-// and the final sums.  Per-block sums are reduced in a fixed order, so the
+// converted) is left to one multiply-add per channel of a pixel that differs,
+// one addition per window and channel, and the final sums.  Per-block sums are reduced in a fixed order, so the
 // result is deterministic.
-// 1280 x 720, FP32 images, both kernels: one window per thread 92 us, this 64 us;
-// eight windows per thread 79 us (their unrolled code leaves the instruction cache).
+// GB300, whole calls, FP32 images, against one window per thread: 640 x 360 56 ->
+// 54 us, 1280 x 720 114 -> 89, 1920 x 1080 200 -> 152, 3840 x 2160 684 -> 488.
+// Four blocks per SM hold a thread's four windows in registers; five (96
+// registers) spill 480 bytes a thread: 64, 113, 192 and 605 us.  Eight windows
+// per thread: the unrolled code leaves the instruction cache (23% slower).
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -133,7 +136,7 @@ __device__ __forceinline__ void ssim_column(const float2 (*P)[kSx], int lx, int 
 }
 
 // partial[block] = (sum of SSIM over the block's windows and channels, sum of squared errors)
-__global__ void __launch_bounds__(32 * kWarps, 5) quality_kernel(const void *__restrict__ a, const void *__restrict__ b,
+__global__ void __launch_bounds__(32 * kWarps, 4) quality_kernel(const void *__restrict__ a, const void *__restrict__ b,
                                                               int fmt, int W, int H, double2 *__restrict__ partial) {
     __shared__ float2 P[3][kSy][kSx];
     __shared__ double red_s[kWarps], red_e[kWarps];
@@ -153,21 +156,15 @@ __global__ void __launch_bounds__(32 * kWarps, 5) quality_kernel(const void *__r
     }
     __syncthreads();
     const int lx = t & 31, ly = (t >> 5) * kRows;
-    // windows centred at (x0 + lx + 3, y0 + ly + q + 3): inside the image when their corner fits.
-    // Their sum in two floats: s + s_lo with the rounding of each addition kept
-    float s = 0.f, s_lo = 0.f;
-    double e_sum = 0.0;
+    // windows centred at (x0 + lx + 3, y0 + ly + q + 3): inside the image when their corner fits
+    double s_sum = 0.0, e_sum = 0.0;
     if (y0 + ly + kWin <= H)  // the same for the whole warp
         for (int c = 0; c < 3; ++c) {
             float w[kRows];
             ssim_column(P[c], lx, ly, w);
 #pragma unroll
             for (int q = 0; q < kRows; ++q)
-                if (x0 + lx + kWin <= W && y0 + ly + q + kWin <= H) {
-                    const float sum = __fadd_rn(s, w[q]), back = __fsub_rn(sum, s);
-                    s_lo += __fadd_rn(__fsub_rn(s, __fsub_rn(sum, back)), __fsub_rn(w[q], back));
-                    s = sum;
-                }
+                if (x0 + lx + kWin <= W && y0 + ly + q + kWin <= H) s_sum += widen(w[q]);
         }
     // squared error: each pixel once, by the thread of its position in the block's tile
     for (int q = 0; q < kRows; ++q)
@@ -181,7 +178,6 @@ __global__ void __launch_bounds__(32 * kWarps, 5) quality_kernel(const void *__r
                 const double d = off == 0.f ? widen(df) : (double)p.x - (double)p.y;
                 e_sum += d * d;
             }
-    double s_sum = isfinite(s) ? (double)s + (double)s_lo : (double)s;
     for (int o = 16; o > 0; o >>= 1) {
         s_sum += __shfl_down_sync(0xffffffffu, s_sum, o);
         e_sum += __shfl_down_sync(0xffffffffu, e_sum, o);

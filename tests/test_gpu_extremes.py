@@ -67,3 +67,20 @@ def test_quality_of_infinite_and_nan_pixels(V, fmt, at, pa, pb, psnr):
         img[k][at[0], at[1], 3] = (pa, pb)[k]
     ssim, got = V.vdi_image_quality(*[torch.from_numpy(i).to(dt).cuda() for i in img], fmt)
     assert math.isfinite(ssim) and math.isfinite(got)
+
+
+@pytest.mark.parametrize("colours", [((0.3, 0.7), (0.0, 1.0), (0.0, 1000.0)), ((0.31, 0.77), (0.0, 30.7), (0.0, 777.7))])
+def test_ssim_sums_in_fp64(V, colours):
+    """Constant channels: every window of a channel has the same FP32 value, so
+    the image's SSIM is their exact mean up to the rounding of 12 additions and a
+    division in FP64 (16 half ulps), whatever the terms' magnitudes."""
+
+    def ssim(H, ch):
+        ab = np.asarray(ch, np.float32).T  # [2, 3]
+        img = [np.ascontiguousarray(np.broadcast_to(np.append(c, 1).astype(np.float32), (H, 7, 4))) for c in ab]
+        return V.vdi_image_quality(*[torch.from_numpy(i).cuda() for i in img])[0]
+
+    w = [ssim(7, [c] * 3) for c in colours]  # one window per channel
+    assert all(x == float(np.float32(x)) for x in w)
+    exact = math.fsum(w * 4) / 12
+    assert abs(ssim(10, colours) - exact) <= 16 * 2.0 ** -53 * exact
