@@ -11,15 +11,15 @@
 //    over the windows and the three channels.
 //  * PSNR = 10 log10(1 / MSE), MSE over every pixel and the three channels.
 // What bounds it: shared-memory reads and issue.  A window needs its 49 pixels
-// twice (mean, then deviations).  A thread takes kRows windows below one
+// twice (mean, then deviations).  A thread takes four windows below one
 // another and reads each row's seven pixels once for all of them, both images
 // of a pixel as one float2, which packed FP32x2 arithmetic sums in one
 // instruction; every window still adds its pixels row by row, left to right.
 // A block's 32 x 16 windows read a 38 x 22 pixel footprint staged in shared
 // memory.  FP64 (a narrow pipe: a third of the time when every difference was
 // converted) is left to one multiply-add per channel of a pixel that differs,
-// one addition per window and channel, and the final sums.  Per-block sums are reduced in a fixed order, so the
-// result is deterministic.
+// one addition per window and channel, and the final sums.  Per-block sums are
+// reduced in a fixed order, so the result is deterministic.
 // GB300, whole calls, FP32 images, against one window per thread: 640 x 360 56 ->
 // 54 us, 1280 x 720 114 -> 89, 1920 x 1080 200 -> 152, 3840 x 2160 684 -> 488.
 // Four blocks per SM hold a thread's four windows in registers; five (96
@@ -39,9 +39,7 @@
 namespace vdi {
 
 constexpr int kWin = 7, kHalf = 3;
-constexpr int kRows = 4, kWarps = 4;                       // windows per thread, warps per block
-constexpr int kTx = 32, kTy = kRows * kWarps;                // window centres per block
-constexpr int kSx = kTx + 2 * kHalf, kSy = kTy + 2 * kHalf;  // staged footprint
+constexpr int kTx = 32, kSx = kTx + 2 * kHalf;  // window centres per block in x, staged pixels
 
 __device__ __forceinline__ float3 load_rgb(const void *img, int fmt, size_t i) {
     if (fmt == 0) {
@@ -85,39 +83,40 @@ __device__ __forceinline__ double widen(float x) {
     return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
 }
 
-// SSIM of the kRows windows whose top-left pixels are P[ly][lx], P[ly + 1][lx], ... (a, b in a float2)
-__device__ __forceinline__ void ssim_column(const float2 (*P)[kSx], int lx, int ly, float (&out)[kRows]) {
-    float2 m[kRows];
+// SSIM of the ROWS windows whose top-left pixels are P[ly][lx], P[ly + 1][lx], ... (a, b in a float2)
+template <int ROWS>
+__device__ __forceinline__ void ssim_column(const float2 (*P)[kSx], int lx, int ly, float (&out)[ROWS]) {
+    float2 m[ROWS];
 #pragma unroll
-    for (int q = 0; q < kRows; ++q) m[q] = make_float2(0.f, 0.f);
+    for (int q = 0; q < ROWS; ++q) m[q] = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int r = 0; r < kRows + kWin - 1; ++r) {
+    for (int r = 0; r < ROWS + kWin - 1; ++r) {
         asm volatile("" ::: "memory");  // one row's pixels in registers at a time
 #pragma unroll
         for (int i = 0; i < kWin; ++i) {
             const float2 v = P[ly + r][lx + i];
 #pragma unroll
-            for (int q = 0; q < kRows; ++q)
+            for (int q = 0; q < ROWS; ++q)
                 if (r >= q && r < q + kWin) m[q] = add_x2(m[q], v);
         }
     }
     const float n = (float)(kWin * kWin);
-    float2 var[kRows];
-    float cov[kRows];
+    float2 var[ROWS];
+    float cov[ROWS];
 #pragma unroll
-    for (int q = 0; q < kRows; ++q) {
+    for (int q = 0; q < ROWS; ++q) {
         m[q] = make_float2(-div_const(m[q].x, n), -div_const(m[q].y, n));
         var[q] = make_float2(0.f, 0.f);
         cov[q] = 0.f;
     }
 #pragma unroll
-    for (int r = 0; r < kRows + kWin - 1; ++r) {  // two-pass: deviations from the window means
+    for (int r = 0; r < ROWS + kWin - 1; ++r) {  // two-pass: deviations from the window means
         asm volatile("" ::: "memory");
 #pragma unroll
         for (int i = 0; i < kWin; ++i) {
             const float2 v = P[ly + r][lx + i];
 #pragma unroll
-            for (int q = 0; q < kRows; ++q)
+            for (int q = 0; q < ROWS; ++q)
                 if (r >= q && r < q + kWin) {
                     const float2 d = add_x2(v, m[q]);
                     var[q] = fma_x2(d, d, var[q]);
@@ -127,7 +126,7 @@ __device__ __forceinline__ void ssim_column(const float2 (*P)[kSx], int lx, int 
     }
     const float C1 = 0.01f * 0.01f, C2 = 0.03f * 0.03f;
 #pragma unroll
-    for (int q = 0; q < kRows; ++q) {
+    for (int q = 0; q < ROWS; ++q) {
         const float ma = -m[q].x, mb = -m[q].y;
         const float vaa = div_const(var[q].x, n - 1.f), vbb = div_const(var[q].y, n - 1.f);
         const float vab = div_const(cov[q], n - 1.f);
@@ -136,10 +135,13 @@ __device__ __forceinline__ void ssim_column(const float2 (*P)[kSx], int lx, int 
 }
 
 // partial[block] = (sum of SSIM over the block's windows and channels, sum of squared errors)
-__global__ void __launch_bounds__(32 * kWarps, 4) quality_kernel(const void *__restrict__ a, const void *__restrict__ b,
-                                                              int fmt, int W, int H, double2 *__restrict__ partial) {
+// BLOCKS: resident blocks per SM
+template <int ROWS, int WARPS, int BLOCKS>
+__global__ void __launch_bounds__(32 * WARPS, BLOCKS)
+    quality_kernel(const void *__restrict__ a, const void *__restrict__ b, int fmt, int W, int H, double2 *__restrict__ partial) {
+    constexpr int kTy = ROWS * WARPS, kSy = kTy + 2 * kHalf;
     __shared__ float2 P[3][kSy][kSx];
-    __shared__ double red_s[kWarps], red_e[kWarps];
+    __shared__ double red_s[WARPS], red_e[WARPS];
     const int t = threadIdx.x;
     const int x0 = blockIdx.x * kTx, y0 = blockIdx.y * kTy;  // first window centre is (x0 + 3, y0 + 3)
     for (int k = t; k < kSx * kSy; k += blockDim.x) {
@@ -155,19 +157,19 @@ __global__ void __launch_bounds__(32 * kWarps, 4) quality_kernel(const void *__r
         P[2][sy][sx] = make_float2(va.z, vb.z);
     }
     __syncthreads();
-    const int lx = t & 31, ly = (t >> 5) * kRows;
+    const int lx = t & 31, ly = (t >> 5) * ROWS;
     // windows centred at (x0 + lx + 3, y0 + ly + q + 3): inside the image when their corner fits
     double s_sum = 0.0, e_sum = 0.0;
     if (y0 + ly + kWin <= H)  // the same for the whole warp
         for (int c = 0; c < 3; ++c) {
-            float w[kRows];
-            ssim_column(P[c], lx, ly, w);
+            float w[ROWS];
+            ssim_column<ROWS>(P[c], lx, ly, w);
 #pragma unroll
-            for (int q = 0; q < kRows; ++q)
+            for (int q = 0; q < ROWS; ++q)
                 if (x0 + lx + kWin <= W && y0 + ly + q + kWin <= H) s_sum += widen(w[q]);
         }
     // squared error: each pixel once, by the thread of its position in the block's tile
-    for (int q = 0; q < kRows; ++q)
+    for (int q = 0; q < ROWS; ++q)
         if (x0 + lx < W && y0 + ly + q < H)
             for (int c = 0; c < 3; ++c) {
                 const float2 p = P[c][ly + q][lx];
@@ -189,13 +191,17 @@ __global__ void __launch_bounds__(32 * kWarps, 4) quality_kernel(const void *__r
     __syncthreads();
     if (t == 0) {
         double s = 0.0, e = 0.0;
-        for (int w = 0; w < kWarps; ++w) {
+        for (int w = 0; w < WARPS; ++w) {
             s += red_s[w];
             e += red_e[w];
         }
         partial[blockIdx.y * gridDim.x + blockIdx.x] = make_double2(s, e);
     }
 }
+
+// Images of fewer 32 x 16 blocks than this take one window per thread: they
+// leave SMs idle either way, and a thread's chain is a quarter as long.
+constexpr int kSmallBlocks = 128;
 
 // one block: sums the per-block partials in a fixed order
 __global__ void quality_reduce_kernel(const double2 *__restrict__ partial, int n, double2 *__restrict__ total) {
@@ -229,12 +235,16 @@ VDI_API vdi_status vdi_image_quality(const void *a, const void *b, int W, int H,
         return fail(VDI_ERR_INVALID_ARG, "image %dx%d: at least 7 x 7 pixels", W, H);
     if (fmt != VDI_F32 && fmt != VDI_F16) return fail(VDI_ERR_INVALID_ARG, "fmt=%d", fmt);
     cudaStream_t st = (cudaStream_t)stream;
-    const dim3 grid(div_up(W, kTx), div_up(H, kTy));
+    const bool small = (long long)div_up(W, kTx) * div_up(H, 16) < kSmallBlocks;
+    const dim3 grid(div_up(W, kTx), div_up(H, small ? 8 : 16));
     const int nb = (int)(grid.x * grid.y);
     double2 *d = nullptr;
     cudaError_t e = cudaMallocAsync((void **)&d, sizeof(double2) * (size_t)(nb + 1), st);
     if (e != cudaSuccess) return cuda_fail(e, "quality scratch");
-    quality_kernel<<<grid, 32 * kWarps, 0, st>>>(a, b, fmt, W, H, d + 1);
+    if (small)
+        quality_kernel<1, 8, 4><<<grid, 256, 0, st>>>(a, b, fmt, W, H, d + 1);
+    else
+        quality_kernel<4, 4, 4><<<grid, 128, 0, st>>>(a, b, fmt, W, H, d + 1);
     e = cudaGetLastError();
     double2 h = make_double2(0.0, 0.0);
     if (e == cudaSuccess) {

@@ -84,3 +84,16 @@ def test_ssim_sums_in_fp64(V, colours):
     assert all(x == float(np.float32(x)) for x in w)
     exact = math.fsum(w * 4) / 12
     assert abs(ssim(10, colours) - exact) <= 16 * 2.0 ** -53 * exact
+
+
+@pytest.mark.parametrize("W,H", [(7, 7), (8, 22), (33, 9), (320, 200), (1024, 48), (256, 256), (513, 129), (700, 300)])
+def test_quality_by_image_size(V, W, H):
+    """One window per thread in images of fewer than 128 blocks of 32 x 16
+    windows, four in larger ones: the oracle's measures on both sides."""
+    from oracle import quality as Q
+
+    rng = np.random.default_rng(W + H)
+    a = rng.uniform(0, 1, (H, W, 4)).astype(np.float32)
+    b = np.clip(a + rng.normal(0, 0.05, a.shape), 0, 1).astype(np.float32)
+    ssim, psnr = V.vdi_image_quality(torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda())
+    assert abs(ssim - Q.ssim(a, b)) < 2e-6 and abs(psnr - Q.psnr(a, b)) < 1e-6
