@@ -813,12 +813,18 @@ static vdi_status make_gen_consts(const vdi_volume *vol, const vdi_tf *tf, const
     // per axis and 2^31 in all, extents and segment widths whose reciprocals
     // and residuals stay clear of under- and overflow, and knots that are 0 or
     // no smaller than 2^-60 (then v - knot is 0 or above 2^-91 for integer
-    // voxels).  Anything else samples by plain divisions.
+    // voxels).  Positions are rounded at the magnitude of the eye's and the
+    // box's coordinates: with their sum at most 2^40 extents per n voxels, the
+    // errors of the few operations behind a position stay below 2^20 voxels and
+    // its voxel coordinate below 2^22, where the mantissa floor holds.
+    // Anything else samples by plain divisions.
     g->fast = vol->nx < (1 << 21) && vol->ny < (1 << 21) && vol->nz < (1 << 21) &&
               (double)vol->nx * vol->ny * vol->nz < 2147483648.0;
     g->unit_ext = 1;
     for (int k = 0; k < 3; ++k) {
         if (!(g->ext[k] >= 0x1p-30f && g->ext[k] <= 0x1p60f)) g->fast = 0;
+        const double n = k == 0 ? vol->nx : k == 1 ? vol->ny : vol->nz;
+        if (!((fabs((double)g->E[k]) + fabs((double)g->bmin[k]) + fabs((double)g->bmax[k])) * n <= 0x1p40 * g->ext[k])) g->fast = 0;
         if (g->ext[k] != 1.f) g->unit_ext = 0;
         g->iext[k] = 1.f / g->ext[k];
     }

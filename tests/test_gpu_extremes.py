@@ -97,3 +97,41 @@ def test_quality_by_image_size(V, W, H):
     b = np.clip(a + rng.normal(0, 0.05, a.shape), 0, 1).astype(np.float32)
     ssim, psnr = V.vdi_image_quality(torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda())
     assert abs(ssim - Q.ssim(a, b)) < 2e-6 and abs(psnr - Q.psnr(a, b)) < 1e-6
+
+
+def far_camera(D):
+    """An eye at (-D, 1/2, 1/2) looking along x at a box one unit across."""
+    view = np.array([[0, 0, 1, -0.5], [0, 1, 0, -0.5], [-1, 0, 0, -D], [0, 0, 0, 1.0]])
+    near, far = D / 2, 2 * D
+    proj = np.zeros((4, 4))
+    proj[0, 0] = proj[1, 1] = 4 * D
+    proj[2, 2], proj[2, 3], proj[3, 2] = -(far + near) / (far - near), -2 * far * near / (far - near), -1.0
+    return view, proj
+
+
+@pytest.mark.parametrize("dtype", [np.uint8, np.uint16, np.float32])
+@pytest.mark.parametrize("log_d", [41, 46, 30])
+@pytest.mark.parametrize("axis", [0, 1])
+def test_sampling_from_a_distant_eye(V, ctx, orc, dtype, log_d, axis):
+    """FP32 positions are up to 2^23 units apart: they fall on either side of the
+    box, up to 2^29 voxels away, and read its first and last voxels, as plain
+    arithmetic does.  (A box half an ulp of the eye's distance away from the
+    origin keeps an interval between its faces.)"""
+    D = 2.0 ** log_d
+    ulp = D * 2.0 ** -23
+    dims = [1, 1, 1]
+    dims[2 - axis] = 128  # along the view, or across it
+    top = 1.0 if dtype == np.float32 else np.iinfo(dtype).max
+    vol = np.zeros(dims, dtype)
+    vol.reshape(-1)[:64] = top
+    kn = np.array([[0, 0.1, 0.2, 0.9, 0.01], [1, 0.9, 0.3, 0.1, 0.02]], np.float32)
+    bmin = np.array([max(ulp / 2 - 0.5, 0.0), 0, 0])
+    bmax = bmin + [1, 1, 1]
+    view, proj = far_camera(D)
+    step = max(ulp / 2.0 ** 12, 1.0)
+    args = (kn, view, proj, 6, 5)
+    ref = orc.dvr(orc.Volume(vol, bmin, bmax), *args, step, step, fp32=True)
+    out = torch.zeros((5, 6, 4), device="cuda")
+    V.vdi_dvr(ctx, torch.from_numpy(vol).cuda(), bmin, bmax, kn, V.camera(view, proj), 6, 5, step, step, out)
+    assert ref[:, 3].min() > 0.5
+    assert np.abs(out.cpu().numpy().reshape(-1, 4) - ref).max() < 1e-5
