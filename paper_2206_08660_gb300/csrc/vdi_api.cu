@@ -602,7 +602,7 @@ VDI_API vdi_status vdi_create(vdi_ctx *ctx, const vdi_desc *desc, const float *r
     const size_t nl = (size_t)desc->w * desc->h, nslot = nl * desc->n_s;
     float *d_rgba = nullptr, *d_depth = nullptr;
     int32_t *d_counts = nullptr;
-    const int32_t *use_counts = counts;  // device counts are read where they are
+    const int32_t *use_counts = counts;  // device counts are read where they are, if 4-byte aligned
     unsigned *d_err = nullptr;
     unsigned h_err = 0;
     if (mem_kind == VDI_MEM_HOST) {
@@ -616,11 +616,12 @@ VDI_API vdi_status vdi_create(vdi_ctx *ctx, const vdi_desc *desc, const float *r
     }
     CK(cudaMallocAsync((void **)&d_err, sizeof(unsigned), st));
     CK(cudaMemsetAsync(d_err, 0, sizeof(unsigned), st));
-    if (!counts || mem_kind == VDI_MEM_HOST) {
+    if (!counts || mem_kind == VDI_MEM_HOST || (reinterpret_cast<uintptr_t>(counts) & 3)) {
         CK(cudaMallocAsync((void **)&d_counts, nl * sizeof(int32_t), st));
         use_counts = d_counts;
         if (counts)
-            CK(cudaMemcpyAsync(d_counts, counts, nl * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+            CK(cudaMemcpyAsync(d_counts, counts, nl * sizeof(int32_t),
+                               mem_kind == VDI_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, st));
         else
             CK(launch_count_leading(d_depth, desc->n_s, (long long)nl, d_counts, st));
     }

@@ -6,7 +6,7 @@ import math
 import numpy as np
 import pytest
 
-import vdi_synth as S
+from helpers import random_case
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -135,3 +135,20 @@ def test_sampling_from_a_distant_eye(V, ctx, orc, dtype, log_d, axis):
     V.vdi_dvr(ctx, torch.from_numpy(vol).cuda(), bmin, bmax, kn, V.camera(view, proj), 6, 5, step, step, out)
     assert ref[:, 3].min() > 0.5
     assert np.abs(out.cpu().numpy().reshape(-1, 4) - ref).max() < 1e-5
+
+
+@pytest.mark.parametrize("offset", [1, 2, 3, 4])
+def test_create_with_unaligned_device_counts(V, ctx, offset):
+    """Device counts at any byte address, as a copy takes them."""
+    case = random_case(37, 21, 5, seed=2)
+    a = case.vdi
+    rgba, depth = torch.from_numpy(a.rgba).cuda(), torch.from_numpy(a.depth).cuda()
+    raw = torch.zeros(4 * a.counts.size + 8, dtype=torch.uint8, device="cuda")
+    counts = raw[offset:offset + 4 * a.counts.size]
+    counts.copy_(torch.from_numpy(np.ascontiguousarray(a.counts, np.int32).view(np.uint8).reshape(-1)))
+    assert counts.data_ptr() % 4 == offset % 4
+    vdi = V.vdi_create(ctx, case.gpu_desc(V, V.VDI_F32), rgba, depth, counts)
+    try:
+        assert np.array_equal(V.vdi_download(vdi, a.w, a.h, a.ns)[2], a.counts)
+    finally:
+        V.vdi_destroy(vdi)
