@@ -7,6 +7,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "vdi_internal.cuh"
 
 namespace vdi {
@@ -103,8 +105,8 @@ __global__ void convert_kernel(const float *__restrict__ rgba, const float *__re
 // a run is looked for from the last one's end on.
 //
 // What bounds it: issue and the depth records of the lists that hold anything.
-// A block takes a row of kGridCols cells (its counts of a slab are one 32-byte
-// run), reads the ranges first and gathers the lists that are not empty; a
+// A block takes a row of up to kGridCols cells (then its counts of a slab are one
+// 32-byte run; launch_grid), reads the ranges first and gathers the lists that are not empty; a
 // thread then walks one list up to its last supersegment, the next pair
 // requested ahead.  Each counter exists kGridCopies times, by lane, since
 // neighbouring lists count in the same slabs.
@@ -112,16 +114,17 @@ __global__ void convert_kernel(const float *__restrict__ rgba, const float *__re
 // block per cell over every slot with a test per slab 136 us, this 50 us.
 constexpr int kGridCols = 8, kGridCopies = 8, kGridChunk = 512;
 
-__global__ void __launch_bounds__(256) grid_kernel(const DevVdi v, uint32_t *__restrict__ grid, float2 *__restrict__ brange) {
+__global__ void __launch_bounds__(256)
+    grid_kernel(const DevVdi v, uint32_t *__restrict__ grid, float2 *__restrict__ brange, int gc) {  // gc: cells per block
     __shared__ int cnt[(kMaxNz + 1) * kGridCols][kGridCopies];
     __shared__ int sum[(kMaxNz + 1) * kGridCols];
     __shared__ float edges[kMaxNz + 1];
     __shared__ unsigned ids[kGridChunk];
     __shared__ int n_ids;
     const int T = v.T, nz = v.nz, t = threadIdx.x;
-    const int cx0 = blockIdx.x * kGridCols, cy = blockIdx.y;
+    const int cx0 = blockIdx.x * gc, cy = blockIdx.y;
     const int x0 = cx0 * T, y0 = cy * T;
-    const int fx = min(kGridCols * T, v.w - x0), fy = min(T, v.h - y0), lists = fx * fy;
+    const int fx = min(gc * T, v.w - x0), fy = min(T, v.h - y0), lists = fx * fy;
     bool ordered = true;
     for (int k = t; k <= nz; k += blockDim.x) {
         edges[k] = v.edges[k];
@@ -191,7 +194,7 @@ __global__ void __launch_bounds__(256) grid_kernel(const DevVdi v, uint32_t *__r
         }
         __syncthreads();
     }
-    const int cols = min(kGridCols, v.gw - cx0);
+    const int cols = min(gc, v.gw - cx0);
     if (any) {
         for (int k = t; k < nz * kGridCols; k += blockDim.x) {
             int s = 0;
@@ -287,11 +290,18 @@ cudaError_t launch_convert(int fmt, const float *rgba, const float *depth, const
     return cudaGetLastError();
 }
 
-// the count grid and the block ranges of a VDI whose depths and list ranges are written
+// The count grid and the block ranges of a VDI whose depths and list ranges are
+// written.  A block takes cells of 64 lists' width in all, at least one: fewer
+// blocks leave SMs idle when cells are large (1920 x 1080 lists of 20 slots, whole
+// call, eight cells per block against these: T = 32 707 -> 430 us, 64 1870 ->
+// 520, 128 6.08 -> 1.09 ms, 256 20.2 -> 3.3 ms; T = 8 and below have eight).  A
+// block of one large cell would also read its ranges alone, so those have their
+// own kernel from T = 64 on.
 cudaError_t launch_grid(const DevVdi &v, uint32_t *grid, float2 *brange, cudaStream_t st) {
-    const bool whole = v.T % kB == 0;
-    grid_kernel<<<dim3(div_up(v.gw, kGridCols), v.gh), 256, 0, st>>>(v, grid, whole ? brange : nullptr);
-    if (!whole) block_range_kernel<<<dim3(div_up(v.bw, 128), v.bh), 128, 0, st>>>(v, brange);
+    const int gc = std::min(std::max(64 / v.T, 1), kGridCols);
+    const bool fused = v.T % kB == 0 && v.T <= 32;
+    grid_kernel<<<dim3(div_up(v.gw, gc), v.gh), 256, 0, st>>>(v, grid, fused ? brange : nullptr, gc);
+    if (!fused) block_range_kernel<<<dim3(div_up(v.bw, 128), v.bh), 128, 0, st>>>(v, brange);
     return cudaGetLastError();
 }
 
