@@ -243,16 +243,19 @@ struct PreviewWarp {
 template <int FMT, int PW, int R>
 __device__ __forceinline__ void preview_queue(const DevVdi &v, const ViewConsts &c, PreviewWarp<R> &S, int &qn, int n) {
     const int lane = threadIdx.x & 31;
+    const int e = qn - n + min(lane, n - 1);
     __syncwarp();
+    const int id = S.owner[e], ray = id & 31;
+    int seed = S.seed[ray];
+    __syncwarp();  // every seed is read before one is written
     if (lane < n) {
-        const int e = qn - n + lane, id = S.owner[e], ray = id & 31;
         const float4 w = S.w[ray], h0 = S.h0[ray], dh = S.dh[ray];
         const int4 u = S.queue[e];
         const CellSamples q = cell_samples(v, c, w, {u.z, __int_as_float(u.x), __int_as_float(u.y)}, (uint32_t)u.w);
         Accum part = {0.f, 0.f, 0.f, 1.f};
-        int seed = S.seed[ray];
         for (int k = 0; k < q.n; ++k) preview_sample<FMT, PW>(v, h0, dh, q, k, seed, part);
-        S.seed[ray] = seed;  // any lane's: a seed only starts the search
+        // lanes on the same ray store in any order, so atomically: a seed only starts the search
+        __nv_atomic_store_n(&S.seed[ray], seed, __NV_ATOMIC_RELAXED, __NV_THREAD_SCOPE_BLOCK);
         S.part[ray][id >> 5] = make_float4(part.r, part.g, part.b, part.T);
     }
     qn -= n;
