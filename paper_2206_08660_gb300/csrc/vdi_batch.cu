@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, 7) batch_preview_kernel(cons
         __syncthreads();  // (next_tile's first barrier keeps them until every warp is done)
         const int local = tile - q.tile_base;
         int lx, ly;
-        preview_offset(warp * kBatchRays, lx, ly);
+        preview_offset<1>(warp * kBatchRays, lx, ly);
         const int px = (local % q.tiles_x) * kBatchCols + lx, py = (local / q.tiles_x) * 4 + ly;
         const bool inside = (threadIdx.x & 31) < kBatchRays && px < q.c.W && py < q.c.H;
         Ray ray = {};

@@ -5,21 +5,24 @@
 // the sample spacing (Eq. 2).  Compositing is associative, so the cells of the
 // count grid that a ray crosses can be composited apart and merged in order.
 //
-// A warp serves R rays, each walked by one lane in rounds of kRoundCells
-// cells.  Cells that hold something go to the warp's queue in shared memory,
-// and the warp takes 32 of them at a time, one per lane, whichever rays they
-// belong to; each composites to a partial result in shared memory, and a
-// round's partials are merged in a fixed balanced tree (so the image does not
-// depend on R).  Early termination is checked once per round.
+// Large launches (march_preview): a warp serves R rays, each walked by one lane
+// in rounds of kRoundCells cells.  Cells that hold something go to the warp's
+// queue in shared memory, and the warp takes 32 of them at a time, one per
+// lane, whichever rays they belong to; each composites to a partial result in
+// shared memory.  Small launches (march_preview_lanes): eight or four lanes per
+// ray, all of them walking it, each taking its cells of a round.  Either way a
+// round's partials are merged in one fixed balanced tree, so the image does
+// not depend on the choice.  Early termination is checked once per round.
 //
 // What bounds it: the latency of dependent gathers (count, list range and
 // depth pair, colour) and issue.  Walking a ray on every lane that serves it
 // cost half the instructions, and empty cells idled the lanes; with the queue
-// a step is taken once and the sampling lanes are full.  Launches with few
-// rays run with fewer rays per warp, which keeps more warps in flight.
-// GB300, whole previews of 1920 x 1080 lists (20 slots, FP16 colour) at 30
-// degrees: 960 x 540 rays 150 -> 119 us, 480 x 270 rays 68 -> 61 us, 1920 x 1080
-// rays 292 -> 254 us.
+// a step is taken once and the sampling lanes are full.  A launch that leaves
+// issue slots free anyway pays for the queue's extra steps between a round's
+// gathers instead: there the lanes walk along, and a round is a fifth shorter.
+// GB300, warm, 1920 x 1080 lists (20 slots, FP16 colour) at 30 degrees, D_R = 2,
+// against several lanes per ray with an older walk and search: 160 x 90 rays 40 ->
+// 29 us, 480 x 270 60 -> 47, 960 x 540 147 -> 112, 1920 x 1080 334 -> 283.
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
@@ -223,9 +226,7 @@ __device__ __forceinline__ void preview_sample(const DevVdi &v, const float4 &h0
     seed = min(k, npairs - 1);
 }
 
-// steps whose counts are requested together: a whole round where latency counts
-// (320 x 180 rays 42 -> 40 us; with 8 rays per warp 5% slower)
-constexpr int walk_batch(int rays) { return rays <= 4 ? kRoundCells : kRoundCells / 2; }
+constexpr int kWalkBatch = kRoundCells / 2;  // steps whose counts are requested together (a whole round: 5% slower)
 
 // A warp's shared memory: its rays, the queue of occupied cells, the partial results.
 template <int R>
@@ -234,7 +235,7 @@ struct PreviewWarp {
     float4 h0[R], dh[R];     // homogeneous clip coordinates of the ray's start, and to its end
     float4 w[R];             // w0, w1, dw, lu of the ray
     int seed[R];             // the slot pair where the ray's last sample ended
-    static constexpr int kQueue = 32 + R * walk_batch(R);  // a batch adds to fewer than 32
+    static constexpr int kQueue = 32 + R * kWalkBatch;  // a batch adds to fewer than 32
     int4 queue[kQueue];  // sa, sb (bits), cell, supersegments there
     int owner[kQueue];   // ray + 32 cell of the round
 };
@@ -262,13 +263,13 @@ __device__ __forceinline__ void preview_queue(const DevVdi &v, const ViewConsts 
     __syncwarp();
 }
 
-// The previews of the R rays of a warp's first R lanes (R in {4, 8, 16}; every
+// The previews of the R rays of a warp's first R lanes (R in {8, 16, 32}; every
 // lane of the warp must call this, lanes without a ray with active = false).
 // edges: the VDI's slab edges in shared memory.
 template <int FMT, int PW, int R>
 __device__ __forceinline__ Accum march_preview(const DevVdi &v, const float *edges, const ViewConsts &c, PreviewWarp<R> &S,
                                                const Ray &r, bool active) {
-    constexpr int B = walk_batch(R);
+    constexpr int B = kWalkBatch;
     static_assert(kRoundCells % B == 0, "whole batches per round");
     const int lane = threadIdx.x & 31;
     if (lane < R) {
@@ -327,12 +328,99 @@ __device__ __forceinline__ Accum march_preview(const DevVdi &v, const float *edg
     return acc;
 }
 
+// The preview of one ray served by L lanes (every lane of the warp must call
+// this, lanes without a ray with active = false).  Each lane walks the ray and
+// takes G consecutive cells of a round.  Returns the composite in every lane.
+template <int FMT, int PW, int L>
+__device__ __forceinline__ Accum march_preview_lanes(const DevVdi &v, const float *edges, const ViewConsts &c, const Ray &r,
+                                                     bool active) {
+    constexpr int G = kRoundCells / L;
+    const int sub = threadIdx.x & (L - 1);
+    const float4 rw = make_float4(r.w0, r.w1, r.dw, r.lu);
+    const float4 dh = make_float4(r.h1.x - r.h0.x, r.h1.y - r.h0.y, r.h1.z - r.h0.z, r.h1.w - r.h0.w);
+    CellWalk w;
+    cell_walk_init(w, v, edges, r, active);
+    Accum acc = {0.f, 0.f, 0.f, 1.f};
+    bool going = active;
+    int seed = 0;
+    const int maxr = (v.gw + v.gh + v.nz + 3 + kRoundCells - 1) / kRoundCells + 1;
+    for (int round = 0; round < maxr && __any_sync(~0u, going); ++round) {
+        CellRec rec[G];
+#pragma unroll
+        for (int i = 0; i < kRoundCells; ++i) {
+            const CellRec cur = cell_walk_next(w, v, edges, r);
+            if (i / G == sub) rec[i % G] = cur;
+        }
+        uint32_t cnt[G], some = 0;
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            cnt[g] = (going && rec[g].sb > rec[g].sa) ? __ldg(v.grid + rec[g].cell) : 0u;
+            some |= cnt[g];
+        }
+        if (__any_sync(~0u, some != 0u)) {
+            Accum part[G];
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                part[g] = {0.f, 0.f, 0.f, 1.f};
+                if (cnt[g]) {
+                    const CellSamples q = cell_samples(v, c, rw, rec[g], cnt[g]);
+                    for (int k = 0; k < q.n; ++k) preview_sample<FMT, PW>(v, r.h0, dh, q, k, seed, part[g]);
+                }
+            }
+#pragma unroll
+            for (int s = 1; s < G; s <<= 1)
+#pragma unroll
+                for (int g = 0; g + s < G; g += 2 * s) part[g] = over(part[g], part[g + s]);
+            Accum x = part[0];
+#pragma unroll
+            for (int off = 1; off < L; off <<= 1) {
+                Accum o;
+                o.r = __shfl_down_sync(~0u, x.r, off, L);
+                o.g = __shfl_down_sync(~0u, x.g, off, L);
+                o.b = __shfl_down_sync(~0u, x.b, off, L);
+                o.T = __shfl_down_sync(~0u, x.T, off, L);
+                if ((sub & (2 * off - 1)) == 0) x = over(x, o);
+            }
+            x.r = __shfl_sync(~0u, x.r, 0, L);
+            x.g = __shfl_sync(~0u, x.g, 0, L);
+            x.b = __shfl_sync(~0u, x.b, 0, L);
+            x.T = __shfl_sync(~0u, x.T, 0, L);
+            if (going) acc = over(acc, x);
+        }
+        if (acc.T <= kErtT || w.s_in >= w.s_end) going = false;
+    }
+    return acc;
+}
+
 // The ray of a warp's lane within a 32 x 8 tile: rays in 8 x 4 patches, a warp
-// on R consecutive ones.  first: the warp's first ray of the tile's 256.
+// on consecutive ones, L lanes each.  first: the warp's first ray of the tile's 256.
+template <int L>
 __device__ __forceinline__ void preview_offset(int first, int &dx, int &dy) {
-    const int i = first + (int)(threadIdx.x & 31), patch = i >> 5;
+    const int i = first + (int)(threadIdx.x & 31) / L, patch = i >> 5;
     dx = (patch & 3) * 8 + (i & 7);
     dy = (patch >> 2) * 4 + ((i >> 3) & 3);
+}
+
+// A block's shared memory for previews of R rays per warp with L lanes each (1:
+// through the queue), and a ray of it
+template <int R, int L>
+struct PreviewShared {
+    float edges[kMaxNz + 1];
+};
+template <int R>
+struct PreviewShared<R, 1> {
+    PreviewWarp<R> warps[kPreviewWarps];
+    float edges[kMaxNz + 1];
+};
+
+template <int FMT, int R, int L>
+__device__ __forceinline__ Accum preview_ray(const DevVdi &v, const ViewConsts &c, PreviewShared<R, L> &sh, const Ray &r,
+                                             bool active) {
+    static_assert(L == 1 || R * L == 32, "a warp's lanes serve its rays");
+    if constexpr (L > 1)
+        return march_preview_lanes<FMT, kPreviewProbe, L>(v, sh.edges, c, r, active);
+    else
+        return march_preview<FMT, kPreviewProbe, R>(v, sh.edges, c, sh.warps[threadIdx.x >> 5], r, active);
 }
 
 }  // namespace vdi

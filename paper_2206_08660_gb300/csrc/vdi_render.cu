@@ -195,55 +195,63 @@ __global__ void __launch_bounds__(256, RenderOccupancy<5>::blocks)
     if (!ready) mbar_wait(&bar, 0);  // no copy into this block's shared memory may outlive it
 }
 
-// Ray-subsampled preview (Section 4.4) with R rays per warp: the blocks of a
-// 32 x 8 tile meeting the box's pixel rectangle (4 R rays each) come first,
-// then the fill blocks of the tiles outside it.  Seven blocks per SM: six (no
-// spills) 5%, eight 15% slower for 960 x 540 rays.
-template <int FMT, int R>
-__global__ void __launch_bounds__(32 * kPreviewWarps, 7) preview_kernel(const ViewConsts c, const DevVdi v, void *out,
-                                                                             int out_fmt) {
+// Ray-subsampled preview (Section 4.4) with R rays per warp and L lanes per ray
+// (1: through the queue).  The blocks of a 32 x 8 tile meeting the box's pixel
+// rectangle (4 R rays each) come first, then the fill blocks of the tiles
+// outside it.  BLOCKS: resident blocks per SM.
+template <int FMT, int R, int L, int BLOCKS>
+__global__ void __launch_bounds__(32 * kPreviewWarps, BLOCKS)
+    preview_kernel(const ViewConsts c, const DevVdi v, void *out, int out_fmt) {
     constexpr int S = 256 / (kPreviewWarps * R);  // blocks per tile
-    __shared__ PreviewWarp<R> warps[kPreviewWarps];
-    __shared__ float edges[kMaxNz + 1];
+    __shared__ PreviewShared<R, L> sh;
     const int nunits = c.tile_w * c.tile_h * S;
     if ((int)blockIdx.x >= nunits) {
         fill_tiles(c, out, out_fmt, nullptr, nullptr, (int)blockIdx.x - nunits);
         return;
     }
-    for (int k = threadIdx.x; k <= v.nz; k += blockDim.x) edges[k] = v.edges[k];
+    for (int k = threadIdx.x; k <= v.nz; k += blockDim.x) sh.edges[k] = v.edges[k];
     __syncthreads();
-    const int tile = (int)blockIdx.x / S, unit = (int)blockIdx.x - tile * S, warp = threadIdx.x >> 5;
+    const int tile = (int)blockIdx.x / S, unit = (int)blockIdx.x - tile * S, lane = threadIdx.x & 31;
     int lx, ly, tx, ty;
-    preview_offset((unit * kPreviewWarps + warp) * R, lx, ly);
+    preview_offset<L>((unit * kPreviewWarps + (int)(threadIdx.x >> 5)) * R, lx, ly);
     tile_of_block(c, tile, tx, ty);
     const int px = tx * 32 + lx, py = ty * 8 + ly;
-    const bool inside = (threadIdx.x & 31) < R && px < c.W && py < c.H;
+    const bool inside = lane < R * L && px < c.W && py < c.H;
     Ray r = {};
     const bool active = inside && setup_ray<false>(c, px, py, v.w, v.h, r);
-    const Accum acc = march_preview<FMT, kPreviewProbe, R>(v, edges, c, warps[warp], r, active);
-    if (inside) store_px(out, out_fmt, (size_t)py * c.W + px, acc);
+    const Accum acc = preview_ray<FMT>(v, c, sh, r, active);
+    if (inside && lane % L == 0) store_px(out, out_fmt, (size_t)py * c.W + px, acc);
 }
 
-template <int FMT, int R>
+template <int FMT, int R, int L, int BLOCKS>
 static cudaError_t launch_preview_r(const ViewConsts &c, const DevVdi &v, void *out, int out_fmt, cudaStream_t st) {
     const int nrect = c.tile_w * c.tile_h, ntiles = div_up(c.W, 32) * div_up(c.H, 8);
     const int grid = nrect * (256 / (kPreviewWarps * R)) + div_up(ntiles - nrect, kFillTiles);
-    preview_kernel<FMT, R><<<grid, 32 * kPreviewWarps, 0, st>>>(c, v, out, out_fmt);
+    preview_kernel<FMT, R, L, BLOCKS><<<grid, 32 * kPreviewWarps, 0, st>>>(c, v, out, out_fmt);
     return cudaGetLastError();
 }
 
-// rays per warp: fewer for launches with few rays, whose time is the longest
-// ray's chain of dependent loads (the image is the same for any count).
-// After an L2 flush, 4 / 8 / 16 rays per warp: 256 x 144 rays 27 / 35 / 35 us,
-// 320 x 180 42 / 51 / 51, 480 x 270 71 / 69 / 76 (on changing inputs 4 is the
-// faster by 1%), 640 x 360 70 / 57 / 58, 960 x 540 176 / 134 / 122, 1920 x 1080
-// 551 / 344 / 254.
+// Lanes per ray and rays per warp by the number of rays (the image is the same
+// for any of them): with few rays a launch takes as long as the longest ray's
+// chain of dependent loads, with many as long as its instructions.  GB300, warm,
+// D_R = 2, 30 degrees, eight lanes per ray / 8 / 16 / 32 rays per warp, on 1920 x
+// 1080 lists of 20 slots (mixing layer) and on 128 x 128 lists of 8 (blobs):
+//    320 x 180 rays     31 / 54 / 72 / 115 us     15 / 19 / 25 / 36
+//    480 x 270          47 / 53 / 72 / 112        21 / 21 / 25 / 33
+//    640 x 360          74 / 72 / 77 / 118        33 / 29 / 25 / 35
+//    960 x 540         145 / 129 / 113 / 137      64 / 49 / 39 / 41
+//   1280 x 720         236 / 201 / 163 / 168     107 / 82 / 55 / 55
+//   1600 x 900         354 / 289 / 222 / 221     162 / 123 / 82 / 73
+//   1920 x 1080        493 / 396 / 293 / 283     230 / 174 / 115 / 96
+// After an L2 flush eight lanes are the faster up to 160,000 rays by more, and
+// the rest is in the same order.
 template <int FMT>
 static cudaError_t launch_preview(const ViewConsts &c, const DevVdi &v, void *out, int out_fmt, cudaStream_t st) {
     const long long rays = (long long)c.W * c.H;
-    if (rays <= 160000) return launch_preview_r<FMT, 4>(c, v, out, out_fmt, st);
-    if (rays <= 300000) return launch_preview_r<FMT, 8>(c, v, out, out_fmt, st);
-    return launch_preview_r<FMT, 16>(c, v, out, out_fmt, st);
+    if (rays <= 160000) return launch_preview_r<FMT, 4, 8, 6>(c, v, out, out_fmt, st);
+    if (rays <= 300000) return launch_preview_r<FMT, 8, 1, 7>(c, v, out, out_fmt, st);
+    if (rays <= 1200000) return launch_preview_r<FMT, 16, 1, 7>(c, v, out, out_fmt, st);
+    return launch_preview_r<FMT, 32, 1, 6>(c, v, out, out_fmt, st);
 }
 
 // Instrumented exact render: marks the VDI words the algorithm reads.
@@ -419,8 +427,8 @@ static cudaError_t launch_m(const ViewConsts &c, const DevVdi &v, void *out, int
                             uint32_t *rs, int warp_shape, bool ert, bool ess, bool blocks, const TileMaps *tm,
                             cudaStream_t st) {
     if (c.d_r > 1) {
-        // previews ignore the search mode and the warp shape (their samples use
-        // a wide probe, several lanes serve a ray); their counters stay zero
+        // previews ignore the search mode and the warp shape (they have their own
+        // search and rays per warp); their counters stay zero
         if (rl) CK_RET(cudaMemsetAsync(rl, 0, sizeof(uint32_t) * c.W * c.H, st));
         if (rs) CK_RET(cudaMemsetAsync(rs, 0, sizeof(uint32_t) * c.W * c.H, st));
         return launch_preview<FMT>(c, v, out, out_fmt, st);
