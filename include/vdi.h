@@ -271,7 +271,7 @@ void vdi_pi_destroy(vdi_pi *pi);
  * Render up to VDI_BATCH_MAX_REQUESTS views of up to VDI_BATCH_MAX_VDIS
  * resident VDIs (of any resolutions, formats, previews) in one batched
  * launch: exact requests are cut into 32x8-pixel tiles and previews (d_r > 1)
- * into 16x4-pixel tiles, 16 rays per warp; each kind forms a queue
+ * into 8x4- or 16x4-pixel tiles, by their number of rays; each kind forms a queue
  * that a persistent grid of (SM count x resident blocks per SM) blocks drains.
  * Each request renders exactly as vdi_render would (the same per-pixel
  * arithmetic, so results do not depend on what else is in the batch).

@@ -2,7 +2,7 @@
 // launch, optionally replayed from a CUDA graph, plus the batch autotuner.
 //
 // Exact requests are cut into 32 x 8 pixel tiles, ray-subsampled previews into
-// 16 x 4 tiles; each kind forms one queue, drained by its own persistent grid
+// 8 x 4 or 16 x 4 tiles; each kind forms one queue, drained by its own persistent grid
 // (SM count x resident blocks per SM) pulling tiles from an atomic counter, so
 // requests of different resolutions, previews and VDIs share the GPU without a
 // launch per view.  Requests with image-space
@@ -30,9 +30,9 @@
 namespace vdi {
 
 constexpr int kMaxBatchReq = VDI_BATCH_MAX_REQUESTS;
-constexpr int kBatchWarps = 4;                               // warps of a preview block
-constexpr int kBatchRays = 16;                                // preview rays per warp
-constexpr int kBatchCols = kBatchWarps * kBatchRays / 4;       // a block's tile: kBatchCols x 4 rays
+// a preview block's warps and tile for R rays per warp, L lanes per ray
+constexpr int batch_warps(int L) { return L > 1 ? 8 : kPreviewWarps; }
+constexpr int batch_cols(int R, int L) { return batch_warps(L) * R / 4; }  // x 4 rows
 constexpr int kMaxBatchVdi = VDI_BATCH_MAX_VDIS;
 
 struct BatchReq {
@@ -45,8 +45,8 @@ struct BatchReq {
 };
 
 // Two tile queues: exact requests (32 x 8 tiles) and ray-subsampled previews
-// (kBatchCols x 4 tiles), each pulled by its own persistent kernel from its own counter.  A
-// request's tile_base counts within its queue; ex_idx / pv_idx list the
+// (batch_cols x 4 tiles), each pulled by its own persistent kernel from its own
+// counter.  A request's tile_base counts within its queue; ex_idx / pv_idx list the
 // requests of each queue in queue order.
 struct BatchParams {
     int n_req, total_tiles, total_ptiles, n_ex, n_pv;
@@ -133,30 +133,29 @@ __global__ void __launch_bounds__(kExactThreads, 1024 / kExactThreads) batch_ren
     }
 }
 
-// Ray-subsampled previews, kBatchRays rays per warp (the same image as the
-// single-view kernels' counts).
-__global__ void __launch_bounds__(32 * kBatchWarps, 7) batch_preview_kernel(const BatchParams P) {
-    __shared__ PreviewWarp<kBatchRays> warps[kBatchWarps];
-    __shared__ float edges[kMaxNz + 1];
-    const int warp = threadIdx.x >> 5;
+// Ray-subsampled previews, R rays per warp and L lanes per ray (1: through the
+// queue); the same image as the single-view kernels'.
+template <int R, int L>
+__global__ void __launch_bounds__(32 * batch_warps(L), L > 1 ? 3 : 7) batch_preview_kernel(const BatchParams P) {
+    __shared__ PreviewShared<R, L> sh;
+    const int lane = threadIdx.x & 31;
     for (;;) {
         int r;
         const int tile = next_tile(P, P.pcounter, P.pv_idx, P.n_pv, P.total_ptiles, r);
         if (tile >= P.total_ptiles) return;
         const BatchReq &q = P.reqs[r];
         const DevVdi &v = P.vdis[q.vdi];
-        for (int k = threadIdx.x; k <= v.nz; k += blockDim.x) edges[k] = v.edges[k];
+        for (int k = threadIdx.x; k <= v.nz; k += blockDim.x) sh.edges[k] = v.edges[k];
         __syncthreads();  // (next_tile's first barrier keeps them until every warp is done)
         const int local = tile - q.tile_base;
         int lx, ly;
-        preview_offset<1>(warp * kBatchRays, lx, ly);
-        const int px = (local % q.tiles_x) * kBatchCols + lx, py = (local / q.tiles_x) * 4 + ly;
-        const bool inside = (threadIdx.x & 31) < kBatchRays && px < q.c.W && py < q.c.H;
+        preview_offset<L>((int)(threadIdx.x >> 5) * R, lx, ly);
+        const int px = (local % q.tiles_x) * batch_cols(R, L) + lx, py = (local / q.tiles_x) * 4 + ly;
+        const bool inside = lane < R * L && px < q.c.W && py < q.c.H;
         Ray ray = {};
         const bool active = inside && setup_ray<false>(q.c, px, py, v.w, v.h, ray);
-        const Accum acc = (v.fmt == 0) ? march_preview<0, kPreviewProbe, kBatchRays>(v, edges, q.c, warps[warp], ray, active)
-                                       : march_preview<1, kPreviewProbe, kBatchRays>(v, edges, q.c, warps[warp], ray, active);
-        if (inside) store_px(q.out, q.out_fmt, (size_t)py * q.c.W + px, acc);
+        const Accum acc = (v.fmt == 0) ? preview_ray<0>(v, q.c, sh, ray, active) : preview_ray<1>(v, q.c, sh, ray, active);
+        if (inside && lane % L == 0) store_px(q.out, q.out_fmt, (size_t)py * q.c.W + px, acc);
     }
 }
 
@@ -195,9 +194,39 @@ static const void *render_fn(int ws) {
 // host side
 // ---------------------------------------------------------------------------
 
+// The preview kernel of a batch by its preview rays, as in the single launch: few
+// rays want the shortest chain, many the fewest instructions.  A tile's fetch
+// and barriers weigh more here, so the lines lie lower and four lanes per ray
+// (tiles twice as large) take the middle.  GB300, a batch of one preview, graph,
+// D_R = 4, eight / four lanes per ray / 16 rays per warp, on 640 x 360 lists of
+// 20 slots (mixing layer) and on 128 x 128 lists of 8 (blobs):
+//    32 x 32 rays   25 / 40 / 60 us      17 / 21 / 27
+//   192 x 144       27 / 41 / 58         17 / 22 / 27
+//   256 x 256       39 / 41 / 59         28 / 24 / 30
+//   480 x 270       47 / 44 / 59         35 / 29 / 31
+//   640 x 360       71 / 60 / 60         54 / 39 / 33
+//   960 x 540      144 / 103 / 80       111 / 72 / 53
+// Requesting the next tile before the current one is rendered is no gain for
+// small batches and 15% to 50% slower for larger ones: the last tiles wait for
+// the blocks that hold them.
+struct BatchPreview {
+    const void *fn;
+    int threads, cols;  // per block, of its tile
+};
+template <int R, int L>
+static BatchPreview batch_preview() {
+    return {(const void *)batch_preview_kernel<R, L>, 32 * batch_warps(L), batch_cols(R, L)};
+}
+static BatchPreview batch_preview_for(long long rays) {
+    if (rays <= 50000) return batch_preview<4, 8>();
+    if (rays <= 200000) return batch_preview<8, 4>();
+    return batch_preview<16, 1>();
+}
+
 struct BatchPlan {
     BatchParams *bp = nullptr;  // host copies (large structs live on the heap)
     UpParams *up = nullptr;
+    BatchPreview preview{};
     size_t scratch_bytes = 0;             // counter + low-resolution images
     std::vector<size_t> lo_offset;        // per request, (size_t)-1 if it renders every pixel
     std::vector<void *> final_out;
@@ -216,6 +245,7 @@ static vdi_status plan_batch(vdi_ctx *ctx, const vdi_request *reqs, int n, Batch
     std::vector<const vdi_t *> vdis;
     size_t off = 256;  // the two queue counters live at offsets 0 and 4
     int tiles = 0, ptiles = 0, up_tiles = 0;
+    long long rays = 0;  // of previews
     pl.lo_offset.assign(n, (size_t)-1);
     pl.final_out.assign(n, nullptr);
     for (int i = 0; i < n; ++i) {
@@ -249,10 +279,8 @@ static vdi_status plan_batch(vdi_ctx *ctx, const vdi_request *reqs, int n, Batch
         }
         q.vdi = vi;
         q.tiles_x = div_up(Wr, 32);
-        if (r.d_r > 1) {  // preview queue: kBatchCols x 4 tiles
-            q.tile_base = ptiles;
-            q.tiles_x = div_up(Wr, kBatchCols);
-            ptiles += q.tiles_x * div_up(Hr, 4);
+        if (r.d_r > 1) {  // preview queue: its tiles below, when its rays are known
+            rays += (long long)Wr * Hr;
             pl.bp->pv_idx[pl.bp->n_pv++] = (unsigned char)i;
         } else {  // exact queue: 32 x 8 tiles in kExactUnits parts
             q.tile_base = tiles;
@@ -278,6 +306,13 @@ static vdi_status plan_batch(vdi_ctx *ctx, const vdi_request *reqs, int n, Batch
             u.tile_base = up_tiles;
             up_tiles += u.tiles_x * div_up(r.H, 8);
         }
+    }
+    pl.preview = batch_preview_for(rays);
+    for (int k = 0; k < pl.bp->n_pv; ++k) {  // preview queue: batch_cols x 4 tiles
+        BatchReq &q = pl.bp->reqs[pl.bp->pv_idx[k]];
+        q.tile_base = ptiles;
+        q.tiles_x = div_up(q.c.W, pl.preview.cols);
+        ptiles += q.tiles_x * div_up(q.c.H, 4);
     }
     pl.bp->n_req = n;
     pl.bp->total_tiles = tiles;
@@ -310,7 +345,7 @@ static int exact_grid(vdi_ctx *ctx, const BatchPlan &pl, int ws, int bps) {
 
 static int preview_grid(vdi_ctx *ctx, const BatchPlan &pl) {
     int occ = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void *)batch_preview_kernel, 32 * kBatchWarps, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, pl.preview.fn, pl.preview.threads, 0);
     return std::min(std::max(1, occ) * ctx->sm_count, std::max(1, pl.bp->total_ptiles));
 }
 
@@ -321,7 +356,7 @@ static cudaError_t enqueue_plain(vdi_ctx *ctx, BatchPlan &pl, int ws, int bps, c
     if (pl.bp->n_ex) e = cudaLaunchKernel(render_fn(ws), dim3(exact_grid(ctx, pl, ws, bps)), dim3(kExactThreads), args, 0, st);
     if (e != cudaSuccess) return e;
     if (pl.bp->n_pv)
-        e = cudaLaunchKernel((const void *)batch_preview_kernel, dim3(preview_grid(ctx, pl)), dim3(32 * kBatchWarps), args, 0, st);
+        e = cudaLaunchKernel(pl.preview.fn, dim3(preview_grid(ctx, pl)), dim3(pl.preview.threads), args, 0, st);
     if (e != cudaSuccess || pl.up->n == 0) return e;
     void *uargs[] = {pl.up};
     return cudaLaunchKernel((const void *)batch_upsample_kernel, dim3(pl.up->total_tiles), dim3(256), uargs, 0, st);
@@ -423,7 +458,7 @@ static vdi_status enqueue_graph(vdi_ctx *ctx, const vdi_request *reqs, int n, Ba
             renders.push_back(ge.render_node);
         }
         if (e == cudaSuccess && pl.bp->n_pv) {
-            const cudaKernelNodeParams kp = kernel_node((const void *)batch_preview_kernel, ge.pgrid, 32 * kBatchWarps, args);
+            const cudaKernelNodeParams kp = kernel_node(pl.preview.fn, ge.pgrid, pl.preview.threads, args);
             e = cudaGraphAddKernelNode(&ge.preview_node, ge.graph, &ms, 1, &kp);
             renders.push_back(ge.preview_node);
         }
@@ -446,7 +481,7 @@ static vdi_status enqueue_graph(vdi_ctx *ctx, const vdi_request *reqs, int n, Ba
             e = cudaGraphExecKernelNodeSetParams(ge.exec, ge.render_node, &kp);
         }
         if (e == cudaSuccess && ge.preview_node) {
-            const cudaKernelNodeParams kp = kernel_node((const void *)batch_preview_kernel, ge.pgrid, 32 * kBatchWarps, args);
+            const cudaKernelNodeParams kp = kernel_node(pl.preview.fn, ge.pgrid, pl.preview.threads, args);
             e = cudaGraphExecKernelNodeSetParams(ge.exec, ge.preview_node, &kp);
         }
         if (e == cudaSuccess && ge.up_node) {

@@ -71,3 +71,40 @@ def test_preview_forms_match_the_oracle(V, ctx, orc, W, H):
     for got in (one, alone):
         frac, _ = check_with_alternatives(got.cpu().numpy(), ref, 0, fl, alts, what=f"preview {W}x{H}")
         assert frac < 0.2
+
+
+def test_a_small_preview_in_a_batch_costs_like_one_alone(V, ctx):
+    """A batch of one small preview (the serving loop's usual batch) against the same
+    preview in a launch of its own, on the device: no more than 1.9 times as long (two
+    launches and a tile queue for one launch); 2.8 times with 16 rays per warp."""
+    n = 128
+    vol = torch.from_numpy(S.value_noise_volume(n, seed=3, dtype=np.uint16)).cuda()
+    bmin, bmax = np.zeros(3), np.ones(3)
+    co = S.orbit_camera(bmin, bmax, 16 / 9, el_deg=20.0)
+    vdi = V.vdi_generate(ctx, vol, bmin, bmax, S.tf_knots("sparse"), V.camera(co.view, co.proj), 640, 360, 20, 0.01, 1 / n,
+                         1 / n, V.VDI_F16)
+    try:
+        W = H = 64
+        cn = S.orbit_camera(bmin, bmax, 1.0, az_deg=30.0, el_deg=20.0)
+        cam = V.camera(cn.view, cn.proj)
+        out = torch.zeros((H, W, 4), device="cuda")
+        req = [V.request(vdi, cam, W, H, 1, 2, out)]
+
+        def us(fn):
+            best = 1e9
+            for _ in range(6):
+                a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+                torch.cuda._sleep(3000000)
+                a.record()
+                for _ in range(20):
+                    fn()
+                b.record()
+                torch.cuda.synchronize()
+                best = min(best, a.elapsed_time(b) / 20 * 1e3)
+            return best
+
+        one = us(lambda: V.vdi_render(vdi, cam, W, H, 1, 2, out))
+        batch = us(lambda: V.vdi_render_batch(ctx, req))
+        assert batch < 1.9 * one
+    finally:
+        V.vdi_destroy(vdi)
