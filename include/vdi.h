@@ -345,7 +345,7 @@ vdi_status vdi_autotune_batch(vdi_ctx *ctx, const vdi_request *reqs, int n, void
 typedef struct vdi_server vdi_server;
 
 typedef struct {
-    size_t budget_bytes;   /* device memory for resident VDIs, unreleased results and preview scratch */
+    size_t budget_bytes;   /* device memory for resident VDIs, unreleased results and scratch */
     int max_batch;         /* requests per launch, 1..VDI_BATCH_MAX_REQUESTS */
     int max_inflight;      /* batches on the device at once (streams), 1..16 */
     int n_slots;           /* resident VDI slots, 1..VDI_BATCH_MAX_VDIS */
@@ -371,7 +371,7 @@ typedef struct {
 typedef struct {
     uint64_t submitted, completed, failed, batches, batched_requests, vdi_installs;
     uint64_t pending, batches_in_flight;
-    size_t bytes_in_use;   /* unreleased images and preview scratch */
+    size_t bytes_in_use;   /* unreleased images, preview scratch, scratch of generations in flight */
     size_t vdi_bytes;      /* live VDI versions and VDIs being generated through the server */
 } vdi_server_counters;
 
@@ -408,7 +408,13 @@ void vdi_server_destroy(vdi_server *s);
  * its samples, so rendering at V_O reproduces the samples' compositing.
  * FP32 arithmetic is IEEE round-to-nearest without fused operations, in a
  * fixed order (supersegment counts and depths are reproducible bit for bit).
- * Also builds the count grid.  Returns after enqueueing on `stream`. */
+ * Also builds the count grid.  Returns after enqueueing on `stream`.
+ * With `adaptive` the ray samples are recorded in device scratch while the work
+ * runs: up to 512 MiB a call (about 0.8 MiB per voxel along a cube's edge at a
+ * step of one voxel and 117,000 lists or more), from a pool of the context that
+ * keeps at most 512 MiB between calls and is given back by vdi_ctx_destroy.
+ * Without that memory, or with too many samples per ray for it, the volume is
+ * sampled again at every gamma tried: the same result in 2 to 15 times the time. */
 enum { VDI_VOL_U8 = 0, VDI_VOL_U16 = 1, VDI_VOL_F32 = 2 };
 
 typedef struct {
@@ -436,7 +442,7 @@ typedef struct {
     int adaptive;        /* 0: gamma = tau for every ray; 1: each ray finds its own gamma by the
                             bisection of Section 3 (Algorithm 3 of the supplement): in [0, sqrt(3)],
                             from 1e-5, until it gets N_S - floor(0.15 N_S) .. N_S supersegments or
-                            the interval is narrower than 1e-4; tau is then ignored */
+                            the interval is narrower than 1e-6; tau is then ignored */
     float *tau_out;      /* DEVICE [h][w] or NULL: the gamma each list used */
 } vdi_gen_params;
 
@@ -448,7 +454,10 @@ vdi_status vdi_generate(vdi_ctx *ctx, const vdi_volume *vol, const vdi_tf *tf, c
  * generation, with its device bytes (vdi_layout_bytes of the parameters)
  * charged to the server's budget before anything is allocated.  VDI_ERR_OOM
  * when they do not fit next to the resident VDIs and unreleased results;
- * other errors as vdi_generate.  Returns after enqueueing. */
+ * other errors as vdi_generate.  An adaptive generation takes scratch of at
+ * most half of what the budget then has left (none: see vdi_generate), which
+ * counts as in use until the generation has finished; views wait for it, VDIs
+ * are accepted as if it were free.  Returns after enqueueing. */
 vdi_status vdi_server_generate(vdi_server *s, int slot, const vdi_volume *vol, const vdi_tf *tf,
                                const vdi_gen_params *params, void *stream);
 

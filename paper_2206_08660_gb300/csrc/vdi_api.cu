@@ -392,6 +392,18 @@ VDI_API vdi_status vdi_ctx_create(int device, vdi_ctx **out) {
         delete c;
         return cuda_fail(e, "cudaStreamCreate");
     }
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    uint64_t keep = kAdaptiveScratch;
+    if ((e = cudaMemPoolCreate(&c->scratch_pool, &props)) != cudaSuccess ||
+        (e = cudaMemPoolSetAttribute(c->scratch_pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+        if (c->scratch_pool) cudaMemPoolDestroy(c->scratch_pool);
+        cudaStreamDestroy(c->free_stream);
+        delete c;
+        return cuda_fail(e, "cudaMemPoolCreate");
+    }
     // VDIs and server images come from the stream-ordered allocator; keep freed
     // blocks in the pool instead of returning them to the driver at every sync
     cudaMemPool_t pool;
@@ -411,6 +423,7 @@ VDI_API void vdi_ctx_destroy(vdi_ctx *ctx) {
         cudaStreamSynchronize(ctx->free_stream);
         cudaStreamDestroy(ctx->free_stream);
     }
+    if (ctx->scratch_pool) cudaMemPoolDestroy(ctx->scratch_pool);  // what is in flight is released when it ends
     delete ctx;
 }
 

@@ -663,31 +663,48 @@ static void launch_adaptive_t(const GenConsts &g, int blocks, float4 *depth, voi
     adaptive_kernel<DT><<<blocks, 32 * kAdaptiveWarps, 0, st>>>(g, depth, colour, range, tau_out, scratch, cap, next);
 }
 
-// Ray-adaptive generation from recorded samples: scratch for the warps in
-// flight from the stream-ordered allocator, at most kAdaptiveScratch bytes.
-// False when rays can have so many samples that too few warps would fit, or
-// when the memory is not to be had; the caller then samples at every pass.
-constexpr size_t kAdaptiveScratch = (size_t)1 << 30;
+// Ray-adaptive generation from recorded samples: the scratch of the warps in
+// flight, at most `limit` bytes.  No blocks when rays can have so many samples
+// that too few warps would fit; the caller then samples at every pass.  (1280 x
+// 720 lists of 256^3 u16 noise, four samples per voxel: 292 blocks 6.4 ms, 146
+// 10.1, 73 19.6, sampled at every pass 18.1; of a 1024^3 u8 mixing layer, two
+// per voxel, 295 blocks 7.0, 147 11.8, sampled 56.7.)
 constexpr int kAdaptiveBlocksPerSm = 6;
 
-static bool launch_adaptive(const GenConsts &g, double diag, int sm_count, float4 *depth, void *colour, float2 *range,
-                            float *tau_out, cudaStream_t st, cudaError_t *e) {
-    *e = cudaSuccess;
-    if (!g.fast) return false;
+struct AdaptivePlan {
+    int cap = 0, blocks = 0;  // entries per lane
+    size_t bytes = 0;
+};
+
+static AdaptivePlan plan_adaptive(const GenConsts &g, double diag, int sm_count, size_t limit) {
+    AdaptivePlan p;
+    if (!g.fast) return p;
     const double most = diag / g.step * 1.001 + 16.0;  // samples of the longest ray, with room for rounding
-    if (!(most < (double)kMaxSamples)) return false;
-    const int cap = (int)most;
-    const size_t per_block = (size_t)cap * 32 * kAdaptiveWarps * sizeof(uint32_t);
+    if (!(most < (double)kMaxSamples)) return p;
+    p.cap = (int)most;
+    const size_t per_block = (size_t)p.cap * 32 * kAdaptiveWarps * sizeof(uint32_t);
     const long long tiles = (long long)div_up(g.w, 8) * div_up(g.h, 4);
-    const long long fit = (long long)(kAdaptiveScratch / per_block);
-    if (fit < sm_count) return false;
-    const int blocks = (int)std::min<long long>(std::min<long long>((long long)sm_count * kAdaptiveBlocksPerSm, fit),
-                                                (tiles + kAdaptiveWarps - 1) / kAdaptiveWarps);
+    const long long fit = limit < 256 ? 0 : (long long)((limit - 256) / per_block);
+    if (4 * fit < 3 * (long long)sm_count) return p;
+    p.blocks = (int)std::min<long long>(std::min<long long>((long long)sm_count * kAdaptiveBlocksPerSm, fit),
+                                        (tiles + kAdaptiveWarps - 1) / kAdaptiveWarps);
+    p.bytes = 256 + per_block * p.blocks;
+    return p;
+}
+
+// False when there is no plan or the memory is not to be had.  The scratch comes
+// from the context's own pool, which keeps at most kAdaptiveScratch bytes between
+// calls (fresh memory on every call would cost as much as the kernel).
+static bool launch_adaptive(const GenConsts &g, const AdaptivePlan &plan, cudaMemPool_t pool, float4 *depth, void *colour,
+                            float2 *range, float *tau_out, cudaStream_t st, cudaError_t *e) {
+    *e = cudaSuccess;
     char *mem = nullptr;
-    if (cudaMallocAsync((void **)&mem, 256 + per_block * blocks, st) != cudaSuccess) {
+    if (!plan.blocks) return false;
+    if (cudaMallocFromPoolAsync((void **)&mem, plan.bytes, pool, st) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
+    const int blocks = plan.blocks, cap = plan.cap;
     unsigned *next = reinterpret_cast<unsigned *>(mem);
     uint32_t *scratch = reinterpret_cast<uint32_t *>(mem + 256);
     *e = cudaMemsetAsync(next, 0, sizeof(unsigned), st);
@@ -710,10 +727,10 @@ static void launch_generate_t(const GenConsts &g, float4 *depth, void *colour, f
     generate_kernel<DT, ADAPTIVE><<<grid, 256, 0, st>>>(g, depth, colour, range, tau_out);
 }
 
-static cudaError_t launch_generate(const GenConsts &g, bool adaptive, double diag, int sm_count, float4 *depth,
-                                   void *colour, float2 *range, float *tau_out, cudaStream_t st) {
+static cudaError_t launch_generate(const GenConsts &g, bool adaptive, const AdaptivePlan &plan, cudaMemPool_t pool,
+                                   float4 *depth, void *colour, float2 *range, float *tau_out, cudaStream_t st) {
     cudaError_t e;
-    if (adaptive && launch_adaptive(g, diag, sm_count, depth, colour, range, tau_out, st, &e)) return e;
+    if (adaptive && launch_adaptive(g, plan, pool, depth, colour, range, tau_out, st, &e)) return e;
     if (adaptive)  // rare (above): the general sampling serves every type
         launch_generate_t<kGeneral, true>(g, depth, colour, range, tau_out, st);
     else switch (g.fast ? g.dtype : kGeneral) {
@@ -838,8 +855,27 @@ static vdi_status make_gen_consts(const vdi_volume *vol, const vdi_tf *tf, const
     return VDI_OK;
 }
 
+static double box_diagonal(const vdi_volume *vol) {
+    double d = 0.0;
+    for (int k = 0; k < 3; ++k) d += (vol->bbox_max[k] - vol->bbox_min[k]) * (vol->bbox_max[k] - vol->bbox_min[k]);
+    return sqrt(d);
+}
+
+size_t vdi::generation_scratch(vdi_ctx *ctx, const vdi_volume *vol, const vdi_tf *tf, const vdi_gen_params *prm, size_t limit) {
+    GenConsts g;
+    if (!prm->adaptive || check_volume_tf_camera(vol, tf, &prm->orig, prm->step) != VDI_OK ||
+        make_gen_consts(vol, tf, &prm->orig, prm->w, prm->h, prm->step, prm->length_unit, &g) != VDI_OK)
+        return 0;
+    return plan_adaptive(g, box_diagonal(vol), ctx->sm_count, limit).bytes;
+}
+
 VDI_API vdi_status vdi_generate(vdi_ctx *ctx, const vdi_volume *vol, const vdi_tf *tf, const vdi_gen_params *prm,
                                 void *stream, vdi_t **out) {
+    return vdi::generate(ctx, vol, tf, prm, kAdaptiveScratch, stream, out);
+}
+
+vdi_status vdi::generate(vdi_ctx *ctx, const vdi_volume *vol, const vdi_tf *tf, const vdi_gen_params *prm,
+                         size_t scratch_limit, void *stream, vdi_t **out) {
     if (!ctx || !vol || !tf || !prm || !out) return fail(VDI_ERR_INVALID_ARG, "NULL argument");
     *out = nullptr;
     vdi_status st_ = check_volume_tf_camera(vol, tf, &prm->orig, prm->step);
@@ -871,9 +907,8 @@ VDI_API vdi_status vdi_generate(vdi_ctx *ctx, const vdi_volume *vol, const vdi_t
     g.nl = v->dv.nl;
     g.fmt = d.colour_fmt;
     cudaStream_t st = (cudaStream_t)stream;
-    double diag = 0.0;
-    for (int k = 0; k < 3; ++k) diag += (vol->bbox_max[k] - vol->bbox_min[k]) * (vol->bbox_max[k] - vol->bbox_min[k]);
-    cudaError_t e = launch_generate(g, prm->adaptive != 0, sqrt(diag), ctx->sm_count, reinterpret_cast<float4 *>(v->depth_mem),
+    const AdaptivePlan plan = plan_adaptive(g, box_diagonal(vol), ctx->sm_count, scratch_limit);
+    cudaError_t e = launch_generate(g, prm->adaptive != 0, plan, ctx->scratch_pool, reinterpret_cast<float4 *>(v->depth_mem),
                                     v->colour_mem, v->range_mem, prm->tau_out, st);
     if (e == cudaSuccess) e = launch_grid(v->dv, v->grid_mem, v->brange_mem, st);
     if (e != cudaSuccess) {

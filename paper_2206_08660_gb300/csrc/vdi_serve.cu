@@ -15,7 +15,8 @@
 //  - every wait is bounded (VDI_ERR_TIMEOUT), errors land on the ticket;
 //  - the memory budget is a device budget: resident VDI versions (including
 //    a replaced one still read by in-flight batches) and a VDI being
-//    generated through the server are charged next to images and scratch.
+//    generated through the server are charged next to images and scratch
+//    (of previews, and of an adaptive generation until it has finished).
 // One scheduler thread owns all CUDA work of the server.
 #include <cuda_runtime.h>
 
@@ -68,6 +69,11 @@ struct Ticket {
     bool released = false;
 };
 
+struct GenScratch {  // of a generation in flight
+    cudaEvent_t done = nullptr;
+    size_t bytes = 0;
+};
+
 struct Batch {
     cudaStream_t stream = nullptr;
     cudaEvent_t done = nullptr;
@@ -90,6 +96,8 @@ struct vdi_server {
     // batches that hold versions, so it outlives them)
     std::atomic<size_t> vdi_bytes{0};
     size_t reserved = 0;  // bytes held for VDIs being generated through the server
+    std::vector<vdi::GenScratch> gen_scratch;  // of adaptive generations not finished yet
+    size_t scratch_bytes = 0;                  // their sum
     std::vector<std::shared_ptr<vdi::VdiVersion>> slots;
     std::vector<vdi::Batch> batches;
     uint64_t next_ticket = 1;
@@ -135,9 +143,24 @@ static void finish(vdi_server *s, uint64_t id, int status) {
     t.scratch = 0;
 }
 
+// release the charge of finished generations' scratch; called with the lock held
+static void reap_scratch(vdi_server *s) {
+    for (size_t i = 0; i < s->gen_scratch.size();) {
+        GenScratch &g = s->gen_scratch[i];
+        if (cudaEventQuery(g.done) == cudaErrorNotReady) {
+            ++i;
+            continue;
+        }
+        cudaEventDestroy(g.done);
+        s->scratch_bytes -= g.bytes;
+        s->gen_scratch.erase(s->gen_scratch.begin() + i);
+    }
+}
+
 // mark finished batches, release their VDI holds; called with the lock held
 static int reap(vdi_server *s) {
     int n = 0;
+    reap_scratch(s);
     for (auto &b : s->batches) {
         if (!b.busy) continue;
         cudaError_t e = cudaEventQuery(b.done);
@@ -187,7 +210,8 @@ static bool launch_one(vdi_server *s) {
             finish(s, id, VDI_ERR_OOM);
             continue;
         }
-        if (s->used + held + need > s->cfg.budget_bytes) break;  // admission by memory: wait for releases
+        // admission by memory: wait for releases (a generation's scratch among them)
+        if (s->used + held + s->scratch_bytes + need > s->cfg.budget_bytes) break;
         std::shared_ptr<VdiVersion> ver = s->slots[r.slot];
         if (!ver->ready_seen) {
             const cudaError_t q = cudaEventQuery(ver->ready);
@@ -368,15 +392,40 @@ VDI_API vdi_status vdi_server_generate(vdi_server *s, int slot, const vdi_volume
     vdi_layout L;
     vdi_status st_ = vdi_layout_bytes(&d, &L);
     if (st_ != VDI_OK) return st_;
-    {  // hold the new VDI's bytes before it is allocated
+    cudaSetDevice(s->ctx->device);
+    size_t scratch = 0;
+    {  // hold the new VDI's bytes, and the generation's scratch, before they are allocated
         std::lock_guard<std::mutex> g(s->mu);
-        if (s->used + s->reserved + vdi_bytes_after_install(s, slot, L.total_bytes) > s->cfg.budget_bytes)
+        reap_scratch(s);
+        const size_t held = s->used + s->reserved + vdi_bytes_after_install(s, slot, L.total_bytes);
+        if (held > s->cfg.budget_bytes)
             return fail(VDI_ERR_OOM, "generating a VDI of %zu bytes exceeds the budget of %zu next to %zu in use",
                         L.total_bytes, s->cfg.budget_bytes, s->used + s->reserved + s->vdi_bytes.load());
+        // scratch takes at most half of what is left, so that views are admitted beside it
+        const size_t left = s->cfg.budget_bytes - held;
+        if (left > s->scratch_bytes)
+            scratch = generation_scratch(s->ctx, vol, tf, params, std::min(kAdaptiveScratch, (left - s->scratch_bytes) / 2));
         s->reserved += L.total_bytes;
+        s->scratch_bytes += scratch;
     }
     vdi_t *v = nullptr;
-    st_ = vdi_generate(s->ctx, vol, tf, params, stream, &v);
+    st_ = generate(s->ctx, vol, tf, params, scratch, stream, &v);
+    if (scratch) {
+        GenScratch q;
+        q.bytes = scratch;
+        const bool follow = st_ == VDI_OK && cudaEventCreateWithFlags(&q.done, cudaEventDisableTiming) == cudaSuccess &&
+                            cudaEventRecord(q.done, (cudaStream_t)stream) == cudaSuccess;
+        if (!follow) {
+            cudaGetLastError();
+            cudaStreamSynchronize((cudaStream_t)stream);
+            if (q.done) cudaEventDestroy(q.done);
+        }
+        std::lock_guard<std::mutex> g(s->mu);
+        if (follow)
+            s->gen_scratch.push_back(q);
+        else
+            s->scratch_bytes -= scratch;
+    }
     if (st_ != VDI_OK) {
         std::lock_guard<std::mutex> g(s->mu);
         s->reserved -= L.total_bytes;
@@ -488,7 +537,8 @@ VDI_API vdi_status vdi_server_stats(vdi_server *s, vdi_server_counters *out) {
     std::lock_guard<std::mutex> g(s->mu);
     *out = s->st;
     out->pending = s->pending.size();
-    out->bytes_in_use = s->used;
+    reap_scratch(s);
+    out->bytes_in_use = s->used + s->scratch_bytes;
     out->vdi_bytes = s->vdi_bytes.load() + s->reserved;
     int busy = 0;
     for (auto &b : s->batches) busy += b.busy;
@@ -513,5 +563,6 @@ VDI_API void vdi_server_destroy(vdi_server *s) {
         if (b.done) cudaEventDestroy(b.done);
     }
     s->slots.clear();
+    for (auto &g : s->gen_scratch) cudaEventDestroy(g.done);
     delete s;
 }
