@@ -53,8 +53,12 @@ struct VdiVersion {  // one VDI installed in a slot, shared by the batches that 
     std::atomic<size_t> *charge = nullptr;  // the server's resident-VDI bytes, while this version lives
     size_t bytes = 0;
     ~VdiVersion() {
+        if (vdi) {
+            // replaced before its producer finished: the memory is freed after that
+            if (ready && !ready_seen) cudaStreamWaitEvent(vdi->ctx->free_stream, ready, 0);
+            free_vdi(vdi);
+        }
         if (ready) cudaEventDestroy(ready);
-        if (vdi) free_vdi(vdi);
         if (charge) charge->fetch_sub(bytes);
     }
 };

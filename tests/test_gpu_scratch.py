@@ -105,3 +105,36 @@ def test_server_charges_adaptive_scratch(V, ctx, spare_mib):
         assert V.vdi_server_stats(srv).bytes_in_use == 0
     finally:
         V.vdi_server_destroy(srv)
+
+
+def test_replaced_vdi_is_freed_after_its_generation(V, ctx):
+    """A slot's VDI replaced while its generation is still queued: its memory is not
+    handed to the images of the views that follow, so the late writes miss them."""
+    n, w, h, ns = 64, 640, 360, 12
+    vol = torch.from_numpy(S.blobs_volume(n, seed=2)).cuda()
+    bmin, bmax = np.zeros(3), np.ones(3)
+    co = S.orbit_camera(bmin, bmax, w / h, el_deg=15.0)
+    kn, cam_o = S.tf_knots("dense"), V.camera(co.view, co.proj)
+    cam = V.camera(*(lambda c: (c.view, c.proj))(S.orbit_camera(bmin, bmax, w / h, az_deg=20.0, el_deg=15.0)))
+    args = (vol, bmin, bmax, kn, cam_o, w, h, ns, 0.02, 1 / n, 1 / n, V.VDI_F32)
+    ref = torch.zeros((h, w, 4), device="cuda")
+    vdi = V.vdi_generate(ctx, *args)
+    V.vdi_render(vdi, cam, w, h, 1, 1, ref)
+    torch.cuda.synchronize()
+    srv = V.vdi_server_create(ctx, budget_bytes=1 << 30, n_slots=1)
+    try:
+        side = torch.cuda.Stream()
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(1_000_000_000)  # half a second
+        V.vdi_server_generate(srv, 0, *args, stream=side)
+        V.vdi_server_set_vdi(srv, 0, vdi)  # the first version dies with its generation queued
+        tickets = [V.vdi_server_submit(srv, V.view_request(0, cam, w, h, out_fmt=V.VDI_F32)) for _ in range(30)]
+        assert all(V.vdi_server_wait(srv, t, 30.0).status == 0 for t in tickets)
+        torch.cuda.synchronize()  # the late generation has run
+        for t in tickets:
+            out = torch.zeros_like(ref)
+            V.vdi_server_read(srv, t, out)
+            assert torch.equal(out, ref)
+            V.vdi_server_release(srv, t)
+    finally:
+        V.vdi_server_destroy(srv)
