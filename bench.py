@@ -896,7 +896,7 @@ def main():
                      zip(wl["frames"], frame_ms.mean(axis=0))},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic, "peak_source": peak_src,
-                     "kernel": "render_kernel (exact path)",
+                     "kernel": "walk_kernel (exact path)",
                      "algorithmic_bytes_per_launch": [int(b) for b in touched],
                      "frac_per_frame": {f"{wl['frames'][i][0]:g}deg": float(tb / (ms / 1e3) / 1e9 / peak)
                                         for i, tb, ms in zip(exact, touched, exact_ms)}},

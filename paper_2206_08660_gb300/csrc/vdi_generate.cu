@@ -409,9 +409,10 @@ __device__ __forceinline__ float2 write_lists(const GenConsts &g, const TfTable 
 // so every interval still to be halved holds more than eight ulps and its
 // midpoint lies strictly inside it.  FP32 with explicit rounding, like the
 // march, so every ray's gamma is reproducible.
-// pass(m): a counting pass into m.  A gamma at which an earlier pass is
-// known to go the same way (Counter; the last pass on either side is kept) needs none: the large gammas the search starts from and its last steps,
-// which move gamma by less than any distance it is compared with, mostly reuse.
+// pass(m): a counting pass into m.  A gamma at which an earlier pass is known
+// to go the same way (Counter; the last pass on either side is kept) needs none:
+// the large gammas the search starts from and its last steps, which move gamma
+// by less than any distance it is compared with, mostly reuse.
 template <class F>
 __device__ __forceinline__ float adaptive_tau(const GenConsts &g, F pass) {
     const int least = g.ns - (15 * g.ns) / 100;
@@ -500,8 +501,9 @@ __global__ void __launch_bounds__(256, 3) generate_kernel(const GenConsts g, flo
 // Measured on GB300, 256^3 u16 -> 720p, N_S = 20, and two frames: 3.30 ms with
 // the volume sampled at every gamma, 1.57 ms recorded, 1.26 ms with the passes
 // that adaptive_tau leaves out (0.96 ms of it this kernel: 0.49 G warp
-// instructions, issue 58%).  Six blocks of four warps per SM; two entries
-// requested together (one 1.31, four 1.40 ms); eight blocks spill (1.25 ms).
+// instructions, issue 58%).  Six blocks of four warps per SM (they spill some 40
+// bytes, eight more, 1.25 ms); two entries requested together (one 1.31, four
+// 1.40 ms).
 constexpr uint32_t kGapEntry = 0xFFC00000u;  // | n: n transparent samples (a NaN; an opaque sample's scalar is none)
 constexpr int kAdaptiveWarps = 4;            // warps per block
 static_assert(kMaxSamples <= 1 << 22, "a gap's length fills the NaN's 22 payload bits");

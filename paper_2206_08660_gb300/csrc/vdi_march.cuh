@@ -443,8 +443,8 @@ __device__ __forceinline__ bool crosses(int o, float f0, float idg) {
 //  * The slots of a pair are walked without index arithmetic, and the next pair
 //    is requested only when the list goes on (back before the range's end).
 // GB300, whole calls on changing inputs: 1080p at 20 degrees of 1920 x 1080
-// lists (20 slots, FP16 colour) 324 -> 239 us, 720p at 15 degrees (256^3 noise,
-// FP32 colour) 237 -> 196 us, 128 x 128 26.7 -> 21.5 us.  Requesting the next list's
+// lists (20 slots, FP16 colour) 332 -> 247 us, 720p at 15 degrees (256^3 noise,
+// FP32 colour) 231 -> 186 us, 128 x 128 24.6 -> 21.9 us.  Requesting the next list's
 // seed pair a step ahead, or the seed before the range test, gains nothing.
 // DIR: the sign of the ray's depth slope.
 template <int FMT, int DIR>
@@ -602,10 +602,11 @@ __device__ __forceinline__ void march_lists(const DevVdi &v, const Ray &r, Accum
 // Views from V_O's own eye (Section 4.1 at zero deviation): every ray projects
 // to one point of V_O's image plane and stays in one list.  A ray that the
 // list walk would treat as exactly one list over s in [0, 1] is composited
-// here with the list's slot pairs (depth and colour records) requested PF at
+// here (early termination, no counters, as in march_lists) with the list's slot pairs (depth and colour records) requested PF at
 // a time, instead of one dependent round trip per pair; its arithmetic is
 // process_list's, so the image is the same.  Any other ray takes the list
-// walk.
+// walk, inlined: the walk's registers make these kernels spill some 100 bytes, but
+// as an out-of-line function it made every original view 7% to 30% slower.
 // ---------------------------------------------------------------------------
 constexpr int kSinglePF = 2;  // slot pairs march_single requests at once
 
@@ -630,10 +631,9 @@ __host__ __device__ __forceinline__ uint32_t staged_bytes(int nsp) {
 // STAGED: the list's range and first kSinglePF slot pairs come from the
 // staged tile `st` (origin x0, y0) when it arrived (non-null) and holds the
 // list, else from global memory; the arithmetic does not change.
-template <int FMT, int MODE, bool ERT, bool STAGED = false>
-__device__ __forceinline__ void march_single(const DevVdi &v, Ray &r, Accum &acc, uint32_t &n_lists,
-                                             uint32_t &n_segs, const StagedTile<FMT> *st = nullptr, int x0 = 0,
-                                             int y0 = 0) {
+template <int FMT, bool STAGED = false>
+__device__ __forceinline__ void march_single(const DevVdi &v, Ray &r, Accum &acc, const StagedTile<FMT> *st = nullptr,
+                                             int x0 = 0, int y0 = 0) {
     constexpr int PF = kSinglePF;
     const int ox = r.ox, oy = r.oy;
     const float dgx = r.dgx, dgy = r.dgy;
@@ -651,7 +651,6 @@ __device__ __forceinline__ void march_single(const DevVdi &v, Ray &r, Accum &acc
     const Seg g = seg_of(r);
     const int li = iy * v.w + ix;
     const float d_in = fmaf(0.f, g.dz, g.z0), d_out = fmaf(1.f, g.dz, g.z0);
-    ++n_lists;
     const int tlx = ix - x0, tly = iy - y0;
     const bool in_tile = STAGED && st != nullptr && (unsigned)tlx < 32u && (unsigned)tly < 8u;
     const int npairs = v.nsp >> 1;
@@ -719,8 +718,7 @@ __device__ __forceinline__ void march_single(const DevVdi &v, Ray &r, Accum &acc
                     }
                     const float da = fmaf(sa, g.dw, g.w1), db = fmaf(sb, g.dw, g.w1);
                     add_piece(acc, col, g.lw * (sb - sa) * rcp_fast(da * db));
-                    ++n_segs;
-                    if (ERT && acc.T <= kErtT) return;
+                    if (acc.T <= kErtT) return;
                 }
                 if (b > d_out) done = true;
             }

@@ -105,8 +105,8 @@ __global__ void __launch_bounds__(256, RenderOccupancy<PATH>::blocks) render_ker
             march_exact_ess<FMT, MODE, ERT>(v, r, acc, nl, nsg);
         else if (PATH == 3)
             march_exact<FMT, MODE, ERT, false, true>(v, r, acc, nl, nsg);
-        else if (PATH == 5)
-            march_single<FMT, MODE, ERT>(v, r, acc, nl, nsg);
+        else if (PATH == 5)  // (launched with Algorithm 2, early termination and no counters)
+            march_single<FMT>(v, r, acc);
         else if (r.dz >= 0.f)  // two copies of the walk, one per depth direction
             march_exact<FMT, MODE, ERT, false, false, 1>(v, r, acc, nl, nsg);
         else
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(32 * kWalkWarps, 32 / kWalkWarps)
 // later slot pairs from global memory.  The wait on the copies is bounded:
 // when it runs out, the rays read global memory, the VDI's status word
 // records it, and the block waits again before it exits.
-template <int FMT, int MODE>
+template <int FMT>
 __global__ void __launch_bounds__(256, RenderOccupancy<5>::blocks)
     staged_single_kernel(const __grid_constant__ TileMaps tm, const ViewConsts c, const DevVdi v, void *out,
                          int out_fmt) {
@@ -189,8 +189,7 @@ __global__ void __launch_bounds__(256, RenderOccupancy<5>::blocks)
     const bool ready = mbar_wait(&bar, 0);
     if (!ready) atomicOr(tm.status, kStatusStageTimeout);
     Accum acc = {0.f, 0.f, 0.f, 1.f};
-    uint32_t nl = 0, nsg = 0;
-    if (hit) march_single<FMT, MODE, true, true>(v, r, acc, nl, nsg, ready ? &st : nullptr, x0, y0);
+    if (hit) march_single<FMT, true>(v, r, acc, ready ? &st : nullptr, x0, y0);
     if (inside) store_px(out, out_fmt, (size_t)py * c.W + px, acc);
     if (!ready) mbar_wait(&bar, 0);  // no copy into this block's shared memory may outlive it
 }
@@ -417,7 +416,7 @@ template <int FMT>
 static cudaError_t launch_staged(const TileMaps &tm, const ViewConsts &c, const DevVdi &v, void *out, int out_fmt,
                                  cudaStream_t st) {
     const int nrect = c.tile_w * c.tile_h, ntiles = div_up(c.W, 32) * div_up(c.H, 8);
-    staged_single_kernel<FMT, kSearchAlg2>
+    staged_single_kernel<FMT>
         <<<nrect + div_up(ntiles - nrect, kFillTiles), 256, 0, st>>>(tm, c, v, out, out_fmt);
     return cudaGetLastError();
 }
@@ -437,13 +436,15 @@ static cudaError_t launch_m(const ViewConsts &c, const DevVdi &v, void *out, int
     if (!ert) return launch_ws<FMT, MODE, false, 0>(c, v, out, out_fmt, rl, rs, warp_shape, st);
     if (rl || rs) return launch_ws<FMT, MODE, true, 0>(c, v, out, out_fmt, rl, rs, warp_shape, st);
     if (ess) return launch_ws<FMT, MODE, true, 1>(c, v, out, out_fmt, rl, rs, warp_shape, st);
-    if (!blocks && c.single_list && MODE == kSearchAlg2) {
-        // the staged kernel's warps cover 32 x 1 pixels (the default here); another
-        // requested shape takes the unstaged one-list kernel with that shape
-        if (tm && warp_shape == 0 && stage_tiles(c, v)) return launch_staged<FMT>(*tm, c, v, out, out_fmt, st);
-        return launch_ws<FMT, MODE, true, 5>(c, v, out, out_fmt, rl, rs, warp_shape, st);
+    if constexpr (MODE == kSearchAlg2) {
+        if (!blocks && c.single_list) {
+            // the staged kernel's warps cover 32 x 1 pixels (the default here); another
+            // requested shape takes the unstaged one-list kernel with that shape
+            if (tm && warp_shape == 0 && stage_tiles(c, v)) return launch_staged<FMT>(*tm, c, v, out, out_fmt, st);
+            return launch_ws<FMT, MODE, true, 5>(c, v, out, out_fmt, rl, rs, warp_shape, st);
+        }
+        if (!blocks) return launch_walk<FMT>(c, v, out, out_fmt, warp_shape, st);
     }
-    if (!blocks && MODE == kSearchAlg2) return launch_walk<FMT>(c, v, out, out_fmt, warp_shape, st);
     if (!blocks) return launch_ws<FMT, MODE, true, 0>(c, v, out, out_fmt, rl, rs, warp_shape, st);
     return launch_ws<FMT, MODE, true, 3>(c, v, out, out_fmt, rl, rs, warp_shape, st);
 }
