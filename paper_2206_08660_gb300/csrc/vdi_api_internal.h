@@ -54,7 +54,8 @@ bool mat4_inv(const double *m, double *out);
 double ndc_to_view_depth(const double *P, double Z);
 void grid_edges(const double *P, int nz, float *edges);
 size_t touch_words(const vdi_t *v);
-// vdi_generate with at most scratch_limit bytes of scratch, and the bytes it will take
+// vdi_generate with at most scratch_limit bytes of scratch, and the bytes it
+// takes under the same limit
 vdi_status generate(vdi_ctx *ctx, const vdi_volume *vol, const vdi_tf *tf, const vdi_gen_params *prm, size_t scratch_limit,
                     void *stream, vdi_t **out);
 size_t generation_scratch(vdi_ctx *ctx, const vdi_volume *vol, const vdi_tf *tf, const vdi_gen_params *prm, size_t limit);

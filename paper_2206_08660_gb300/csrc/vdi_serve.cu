@@ -397,7 +397,7 @@ VDI_API vdi_status vdi_server_generate(vdi_server *s, int slot, const vdi_volume
     vdi_status st_ = vdi_layout_bytes(&d, &L);
     if (st_ != VDI_OK) return st_;
     cudaSetDevice(s->ctx->device);
-    size_t scratch = 0;
+    size_t scratch = 0, limit = 0;
     {  // hold the new VDI's bytes, and the generation's scratch, before they are allocated
         std::lock_guard<std::mutex> g(s->mu);
         reap_scratch(s);
@@ -407,13 +407,13 @@ VDI_API vdi_status vdi_server_generate(vdi_server *s, int slot, const vdi_volume
                         L.total_bytes, s->cfg.budget_bytes, s->used + s->reserved + s->vdi_bytes.load());
         // scratch takes at most half of what is left, so that views are admitted beside it
         const size_t left = s->cfg.budget_bytes - held;
-        if (left > s->scratch_bytes)
-            scratch = generation_scratch(s->ctx, vol, tf, params, std::min(kAdaptiveScratch, (left - s->scratch_bytes) / 2));
+        if (left > s->scratch_bytes) limit = std::min(kAdaptiveScratch, (left - s->scratch_bytes) / 2);
+        scratch = generation_scratch(s->ctx, vol, tf, params, limit);
         s->reserved += L.total_bytes;
         s->scratch_bytes += scratch;
     }
     vdi_t *v = nullptr;
-    st_ = generate(s->ctx, vol, tf, params, scratch, stream, &v);
+    st_ = generate(s->ctx, vol, tf, params, limit, stream, &v);  // takes `scratch` bytes
     if (scratch) {
         GenScratch q;
         q.bytes = scratch;

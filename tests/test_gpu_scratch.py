@@ -138,3 +138,34 @@ def test_replaced_vdi_is_freed_after_its_generation(V, ctx):
             V.vdi_server_release(srv, t)
     finally:
         V.vdi_server_destroy(srv)
+
+
+def test_server_generates_small_vdis_from_recorded_samples(V, ctx):
+    """A VDI of fewer tiles than the GPU holds warps takes little scratch, which the
+    server grants: its generation takes as long as vdi_generate's (sampled at every
+    gamma it would take some six times as long)."""
+    n, w, h, ns = 256, 64, 64, 20
+    vol = torch.from_numpy(S.value_noise_volume(n, seed=5, dtype=np.uint16)).cuda()
+    bmin, bmax = np.zeros(3), np.ones(3)
+    co = S.orbit_camera(bmin, bmax, 1.0, el_deg=20.0)
+    args = (vol, bmin, bmax, S.tf_knots("sparse"), V.camera(co.view, co.proj), w, h, ns, 0.0, 1 / n, 1 / n, V.VDI_F32)
+    srv = V.vdi_server_create(ctx, budget_bytes=1 << 30, n_slots=1)
+    try:
+        side = torch.cuda.Stream()
+
+        def ms(call):
+            best = 1e9
+            for _ in range(5):
+                a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+                a.record(side)
+                call()
+                b.record(side)
+                torch.cuda.synchronize()
+                best = min(best, a.elapsed_time(b))
+            return best
+
+        direct = ms(lambda: V.vdi_destroy(V.vdi_generate(ctx, *args, stream=side, adaptive=True)))
+        served = ms(lambda: V.vdi_server_generate(srv, 0, *args, stream=side, adaptive=True))
+        assert served < 2.5 * direct, (served, direct)
+    finally:
+        V.vdi_server_destroy(srv)
